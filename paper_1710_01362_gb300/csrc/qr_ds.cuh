@@ -11,127 +11,10 @@
 // modes' contractions.  The scalar reflector arithmetic (square roots, divisions, the
 // triangular factor T) stays in FP64.
 //
-// Error-free transformations: TwoSum (Knuth: s + e = a + b exactly) and TwoProduct through
-// the fused multiply-add (p + e = a b exactly); the _rn intrinsics keep the compiler from
-// contracting or reassociating them.  Products accumulate as a running float sum plus a
-// float sum of all rounding errors, renormalised once at the end (the compensated dot
-// product of Ogita, Rump and Oishi, SIAM J. Sci. Comput. 26 (2005), with double-single
-// inputs).
+// The arithmetic is in ds.cuh.
 //
 // A value below 2^-126 (about 1.2e-38) is zero here, so a Householder head below it counts as
 // zero (phase 1), where the FP64 path draws that line at 1e-280.
-
-// Conversions by integer arithmetic on the bit patterns (the FP64 <-> FP32 conversion
-// instructions run on the narrow FP64 pipe).  ds_from: the head is the double rounded to
-// nearest-even float (from the 29 dropped significand bits), the tail the exact remainder
-// rounded to a float, scaled by a power of two; values below 2^-126 give zero, values beyond
-// FP32's range take the conversion instruction.  Identical to h = (float) x,
-// l = (float) (x - h) for |x| >= 2^-74.
-__device__ __forceinline__ float magic_i2f(int n) {  // exact for |n| < 2^22
-  return __uint_as_float(0x4B400000u + (unsigned)n) - 12582912.0f;
-}
-__device__ __forceinline__ float2 ds_from(double x) {
-  const unsigned hi32 = (unsigned)__double2hiint(x), lo32 = (unsigned)__double2loint(x);
-  const int e = (int)((hi32 >> 20) & 0x7FFu);
-  if (e < 897) return make_float2(0.f, 0.f);
-  if (e > 1149) return make_float2(__double2float_rn(x), 0.f);
-  unsigned fb = (hi32 & 0x80000000u) | ((unsigned)(e - 896) << 23) | ((hi32 & 0xFFFFFu) << 3) | (lo32 >> 29);
-  const unsigned rest = lo32 & 0x1FFFFFFFu;
-  const unsigned up = (rest > 0x10000000u) || (rest == 0x10000000u && (fb & 1u));
-  fb += up;  // a carry into the exponent field is the correct rounding
-  const int lrem = (int)rest - (int)(up << 29);  // x - h in units of 2^(e - 1075)
-  float l = __fmaf_rn(magic_i2f(lrem >> 14), 16384.0f, magic_i2f(lrem & 0x3FFF));
-  const int se = e - 948;
-  l = se >= 1 ? __fmul_rn(l, __uint_as_float((unsigned)se << 23))
-              : __fmul_rn(__fmul_rn(l, 5.421010862427522e-20f), __uint_as_float((unsigned)(se + 64) << 23));
-  if (hi32 & 0x80000000u) l = -l;
-  return make_float2(__uint_as_float(fb), l);
-}
-// float -> double by the bit pattern (zero and normal floats; others by the instruction)
-__device__ __forceinline__ double f2d_bits(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned ef = (u >> 23) & 0xFFu;
-  if ((u << 1) == 0u) return __hiloint2double((int)(u & 0x80000000u), 0);
-  if (ef == 0u || ef == 255u) return (double)f;
-  return __hiloint2double((int)((u & 0x80000000u) | ((ef + 896u) << 20) | ((u & 0x7FFFFFu) >> 3)), (int)((u & 7u) << 29));
-}
-__device__ __forceinline__ double ds_to(float2 a) { return f2d_bits(a.x) + f2d_bits(a.y); }
-// s + t renormalised to a head and a tail (exact when |s| >= |t|)
-__device__ __forceinline__ float2 ds_quick(float s, float t) {
-  const float h = __fadd_rn(s, t);
-  return make_float2(h, __fsub_rn(t, __fsub_rn(h, s)));
-}
-__device__ __forceinline__ float2 ds_add(float2 a, float2 b) {
-  const float s = __fadd_rn(a.x, b.x);
-  const float v = __fsub_rn(s, a.x);
-  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, v)), __fsub_rn(b.x, v));
-  return ds_quick(s, __fadd_rn(e, __fadd_rn(a.y, b.y)));
-}
-__device__ __forceinline__ float2 ds_neg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 ds_re(float4 z) { return make_float2(z.x, z.y); }
-__device__ __forceinline__ float2 ds_im(float4 z) { return make_float2(z.z, z.w); }
-__device__ __forceinline__ float4 ds_c(float2 re, float2 im) { return make_float4(re.x, re.y, im.x, im.y); }
-__device__ __forceinline__ float4 ds_cfrom(double2 z) { return ds_c(ds_from(z.x), ds_from(z.y)); }
-__device__ __forceinline__ double2 ds_cto(float4 z) { return make_double2(ds_to(ds_re(z)), ds_to(ds_im(z))); }
-
-struct DsAcc {
-  float s, c;  // running sum and the sum of its rounding errors
-  __device__ __forceinline__ void init(float2 a) {
-    s = a.x;
-    c = a.y;
-  }
-  __device__ __forceinline__ void mac(float2 x, float2 y) {  // += x y (the lo*lo term is below the format)
-    const float p = __fmul_rn(x.x, y.x);
-    float e = __fmaf_rn(x.x, y.x, -p);
-    e = __fmaf_rn(x.x, y.y, e);
-    e = __fmaf_rn(x.y, y.x, e);
-    const float t = __fadd_rn(s, p);
-    const float v = __fsub_rn(t, s);
-    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(p, v)), e));
-    s = t;
-  }
-  __device__ __forceinline__ float2 val() const { return ds_quick(s, c); }
-};
-
-// complex accumulators: (ar, ai) += conj(v) w, and (ar, ai) += a b
-__device__ __forceinline__ void ds_conj_mac(DsAcc& ar, DsAcc& ai, float4 v, float4 w) {
-  ar.mac(ds_re(v), ds_re(w));
-  ar.mac(ds_im(v), ds_im(w));
-  ai.mac(ds_re(v), ds_im(w));
-  ai.mac(ds_neg(ds_im(v)), ds_re(w));
-}
-__device__ __forceinline__ void ds_cmac(DsAcc& ar, DsAcc& ai, float4 a, float4 b) {
-  ar.mac(ds_re(a), ds_re(b));
-  ar.mac(ds_neg(ds_im(a)), ds_im(b));
-  ai.mac(ds_re(a), ds_im(b));
-  ai.mac(ds_im(a), ds_re(b));
-}
-
-__device__ __forceinline__ float2 shfl_xor_ds(float2 v, int o) {
-  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
-}
-
-// warp_reduce_t for double-single values: lane L returns the total of value
-// warp_reduce_vid<V>(L)
-template <int V>
-__device__ __forceinline__ float2 warp_reduce_ds_t(float2* v) {
-  const int lane = threadIdx.x & 31;
-  int off = 16;
-#pragma unroll
-  for (int n = V; n > 1; n >>= 1, off >>= 1) {
-    const bool hi = (lane & off) != 0;
-#pragma unroll
-    for (int i = 0; i < n / 2; ++i) {
-      const float2 send = hi ? v[i] : v[i + n / 2];
-      const float2 keep = hi ? v[i + n / 2] : v[i];
-      v[i] = ds_add(keep, shfl_xor_ds(send, off));
-    }
-  }
-  float2 t = v[0];
-#pragma unroll
-  for (; off > 0; off >>= 1) t = ds_add(t, shfl_xor_ds(t, off));
-  return t;
-}
 
 // team_reduce_vec with double-single values and sums (same buffers, same protocol: callers
 // alternate between two `mine` buffers; one cluster barrier per call on cluster teams)
@@ -139,7 +22,7 @@ __device__ void team_reduce_vec_ds(Team& tm, const float2* mine, float2* out, in
   __syncthreads();
   cg::cluster_group cl = cg::this_cluster();
   if (tm.kind == TEAM_CLUSTER) {
-    cl.sync();
+    if (tm.size > 1) cl.sync();
     for (int k = threadIdx.x; k < nval; k += NT) {
       float2 a[16];
 #pragma unroll

@@ -20,6 +20,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "ds.cuh"
 #include "tc.cuh"
 
 namespace cg = cooperative_groups;
@@ -58,6 +59,10 @@ __device__ __forceinline__ typename C2<T>::t cvt(double2 v) {
   r.x = (T)v.x;
   r.y = (T)v.y;
   return r;
+}
+template <>
+__device__ __forceinline__ float2 cvt<float>(double2 v) {  // no conversion on the narrow FP64 pipe
+  return make_float2(d2f_bits(v.x), d2f_bits(v.y));
 }
 template <typename T>
 __device__ __forceinline__ typename C2<T>::t cvt(float2 v) {
@@ -147,7 +152,10 @@ __device__ void grid_sync(Ctl* ctl, long long spin_limit) {
 
 __device__ __forceinline__ void team_sync(Team& tm) {
   if (tm.kind == TEAM_CLUSTER) {
-    cg::this_cluster().sync();
+    if (tm.size > 1)
+      cg::this_cluster().sync();
+    else
+      __syncthreads();  // a cluster barrier costs 450 cycles even for one CTA
   } else {
     grid_sync(tm.ctl, tm.spin_limit);
   }
@@ -200,72 +208,82 @@ __device__ __forceinline__ double warp_reduce_t(double* v) {
   return t;
 }
 
-// All-reduce of nv per-thread values over the team (up to four per barrier).  Deterministic
-// and identical on every CTA.  Inside a CTA the 256 values go through shared memory to warp
-// 0, which adds them in a fixed tree (7 additions per lane, then one transposing butterfly
-// for all values, instead of a butterfly per value on every warp: the additions run on the
-// narrow FP64 pipe).  Cluster teams push each CTA's totals into every peer's shared memory
-// before the cluster barrier, so that after it the sums come from local shared memory; the
-// grid team goes through global memory.
-static_assert(NT == 256, "team_allreduce assumes 256 threads per CTA");
-__device__ void team_allreduce4(Team& tm, double* v, int nv) {
-  __shared__ double s_all[4][NT];
-  __shared__ double s_out[4];
-  __shared__ double s_recv[2][16][4];  // [parity][source rank][value] (cluster teams, <= 16 CTAs)
+// All-reduce of NV <= 4 per-thread values over the team.  Deterministic and identical on every
+// CTA.  Inside a CTA the 256 values go through shared memory to warp 0, which adds them in a
+// fixed tree (7 additions per lane, then one transposing butterfly for all values, instead of a
+// butterfly per value on every warp: a warp's FP64 addition holds the SM's FP64 unit for about
+// 20 cycles whatever its lanes do).  Cluster teams push each CTA's totals into every peer's
+// shared memory before the cluster barrier, so that after it the sums come from local shared
+// memory; the grid team goes through global memory.  `fin` runs on thread 0 with the totals
+// before the last block barrier: scalars derived from them are computed once and read from
+// shared memory (a square root that all eight warps repeat costs 2500 cycles).
+static_assert(NT == 256, "team_reduce assumes 256 threads per CTA");
+__shared__ double s_all[4][NT];
+__shared__ double s_recv[2][16][4];  // [parity][source rank][value] (cluster teams, <= 16 CTAs)
+template <int NV>
+__device__ __noinline__ void team_total(Team& tm, const double* v, double* tot) {  // totals on warp 0
+  static_assert(NV <= 4, "up to four values");
+  constexpr int NB = NV == 1 ? 1 : (NV == 2 ? 2 : 4);  // values of the butterfly
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) s_all[i][threadIdx.x] = i < nv ? v[i] : 0.0;
+  for (int i = 0; i < NV; ++i) s_all[i][threadIdx.x] = v[i];
   __syncthreads();
-  double tot[4] = {0.0, 0.0, 0.0, 0.0};  // this CTA's totals (warp 0, every lane)
-  if (warp == 0) {
-    double t[4];
+  double t[NB];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < NB; ++i) t[i] = 0.0;
+  if (warp == 0) {  // this CTA's totals
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
       const double* a = s_all[i];
       t[i] = ((a[lane] + a[lane + 32]) + (a[lane + 64] + a[lane + 96])) +
              ((a[lane + 128] + a[lane + 160]) + (a[lane + 192] + a[lane + 224]));
     }
-    const double r = warp_reduce_t<4>(t);  // lanes 0, 8, 16, 24: values 0..3
+    const double r = warp_reduce_t<NB>(t);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) tot[i] = __shfl_sync(0xffffffffu, r, 8 * i);
+    for (int i = 0; i < NV; ++i) tot[i] = __shfl_sync(0xffffffffu, r, i * (32 / NB));
   }
   if (tm.kind == TEAM_CLUSTER) {
-    cg::cluster_group cl = cg::this_cluster();
-    if (warp == 0 && lane < tm.size) {
-      double* dst = cl.map_shared_rank(&s_recv[tm.parity][tm.rank][0], lane);
+    if (tm.size > 1) {
+      cg::cluster_group cl = cg::this_cluster();
+      if (warp == 0 && lane < tm.size) {
+        double* dst = cl.map_shared_rank(&s_recv[tm.parity][tm.rank][0], lane);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) dst[i] = tot[i];
-    }
-    cl.sync();
-    if (warp == 0) {
-      double t[4];
+        for (int i = 0; i < NV; ++i) dst[i] = tot[i];
+      }
+      cl.sync();
+      if (warp == 0) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) t[i] = lane < tm.size ? s_recv[tm.parity][lane][i] : 0.0;
-      const double r = warp_reduce_t<4>(t);
-      if ((lane & 7) == 0) s_out[lane >> 3] = r;
+        for (int i = 0; i < NV; ++i) t[i] = lane < tm.size ? s_recv[tm.parity][lane][i] : 0.0;
+        const double r = warp_reduce_t<NB>(t);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) tot[i] = __shfl_sync(0xffffffffu, r, i * (32 / NB));
+      }
     }
   } else {
     double* buf = tm.red + (long long)tm.parity * tm.red_stride;
     if (threadIdx.x == 0)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) buf[tm.rank * 4 + i] = tot[i];
+      for (int i = 0; i < NV; ++i) buf[tm.rank * 4 + i] = tot[i];
     team_sync(tm);
     if (warp == 0) {
-      double t[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int i = 0; i < NB; ++i) t[i] = 0.0;
       for (int r = lane; r < tm.size; r += 32)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) t[i] += buf[r * 4 + i];
-      const double r = warp_reduce_t<4>(t);
-      if ((lane & 7) == 0) s_out[lane >> 3] = r;
+        for (int i = 0; i < NV; ++i) t[i] += buf[r * 4 + i];
+      const double r = warp_reduce_t<NB>(t);
+#pragma unroll
+      for (int i = 0; i < NV; ++i) tot[i] = __shfl_sync(0xffffffffu, r, i * (32 / NB));
     }
   }
-  __syncthreads();
-  for (int i = 0; i < nv; ++i) v[i] = s_out[i];
   tm.parity ^= 1;
 }
-
-__device__ void team_allreduce(Team& tm, double* v, int nv) {
-  for (int i0 = 0; i0 < nv; i0 += 4) team_allreduce4(tm, v + i0, nv - i0 < 4 ? nv - i0 : 4);
+template <int NV, typename F>
+__device__ __forceinline__ void team_reduce(Team& tm, const double* v, F&& fin) {
+  double tot[NV];
+  team_total<NV>(tm, v, tot);
+  if (threadIdx.x == 0) fin(tot);
+  __syncthreads();
 }
 
 // Multi-value all-reduce: every CTA has written nval partial doubles at
@@ -575,120 +593,18 @@ __device__ __forceinline__ typename C2<T>::t apply_stage2_at(const KernelParams&
   return acc;
 }
 
-// ------------------------------------------------------------------ tridiagonal exponential
-// u = exp(-i s T) e_0 for the real symmetric tridiagonal T (diag a[0..m), off-diagonal
-// b[1..m) with b[k] coupling k-1 and k), by a Chebyshev expansion on the Gershgorin
-// interval: exp(-i z X) = J_0(z) + 2 sum_n (-i)^n J_n(z) T_n(X), X = (T - c)/R, z = s R.
-// Runs on one warp (lane k holds component k, m <= 32); FP64 throughout.
-__device__ __noinline__ void texp_warp(const double* a, const double* b, int m, double s, double* ure, double* uim) {
-  const int lane = threadIdx.x & 31;
-  const bool on = lane < m;
-  double ak = on ? a[lane] : 0.0;
-  double bk = (on && lane > 0) ? b[lane] : 0.0;
-  double bk1 = (lane + 1 < m) ? b[lane + 1] : 0.0;
-  double lo = on ? ak - fabs(bk) - fabs(bk1) : 1e300;
-  double hi = on ? ak + fabs(bk) + fabs(bk1) : -1e300;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-  }
-  lo = __shfl_sync(0xffffffffu, lo, 0);
-  hi = __shfl_sync(0xffffffffu, hi, 0);
-  const double c = 0.5 * (hi + lo);
-  double R = 0.5 * (hi - lo);
-  double vre = (lane == 0) ? 1.0 : 0.0, vim = 0.0;  // current vector (complex)
-  if (R > 0.0) {
-    // sub-steps so that |z| <= 8 per Chebyshev expansion
-    double zt = fabs(s) * R;
-    if (!(zt < 1e4)) zt = 0.0;  // non-finite input: the caller reports it
-    int nsub = (int)ceil(zt / 8.0);
-    if (nsub < 1) nsub = 1;
-    const double z = s * R / nsub;     // signed
-    const double az = fabs(z);
-    // truncation: the last coefficient ~ 2 (|z|/2)^K / K! below 1e-17
-    int K = 1;
-    {
-      double term = 1.0;
-      while (K < 64 && (term > 1e-18 || K < (int)az + 2)) {
-        term *= 0.5 * az * c_inv[K];
-        ++K;
-      }
-    }
-    // Bessel J_n(|z|) for n = lane and lane + 32 via the power series in Horner form
-    double J[2];
-    const double y = -0.25 * az * az;
-    int jmax = (int)(3.0 * az + 8.0);
-    if (jmax > 24) jmax = 24;
-    for (int h = 0; h < 2; ++h) {
-      const int n = lane + 32 * h;
-      double acc = 1.0;
-      if (n < K) {
-        for (int j = jmax; j >= 1; --j) acc = fma(acc * y, c_inv[j] * c_inv[j + n], 1.0);
-        J[h] = acc * pow(0.5 * az, (double)n) * c_invfact[n];
-      } else {
-        J[h] = 0.0;
-      }
-    }
-    const double dk = on ? (ak - c) / R : 0.0;
-    const double ek = on ? bk / R : 0.0;
-    const double fk = on ? bk1 / R : 0.0;
-    for (int sub = 0; sub < nsub; ++sub) {
-      // Chebyshev on the complex vector v: w = sum_n coef_n T_n(X) v with real T_n
-      double t0r = vre, t0i = vim;
-      double accr = 0.0, acci = 0.0;
-      double tmr = 0.0, tmi = 0.0;   // T_{n-1} v
-      double tr = t0r, ti = t0i;     // T_n v
-      for (int n = 0; n < K; ++n) {
-        const double Jn = __shfl_sync(0xffffffffu, J[n >> 5], n & 31);
-        double cr, ci;  // coef_n = (n ? 2 : 1) (-i sgn(z))^n J_n(|z|)
-        const double w = (n ? 2.0 : 1.0) * Jn;
-        const int q = n & 3;
-        const bool neg = z < 0.0;
-        // (-i)^n for z > 0; (+i)^n for z < 0
-        if (q == 0) { cr = w; ci = 0.0; }
-        else if (q == 2) { cr = -w; ci = 0.0; }
-        else if ((q == 1) != neg) { cr = 0.0; ci = -w; }
-        else { cr = 0.0; ci = w; }
-        accr = fma(cr, tr, fma(-ci, ti, accr));
-        acci = fma(cr, ti, fma(ci, tr, acci));
-        // next Chebyshev vector
-        double trl = __shfl_up_sync(0xffffffffu, tr, 1), til = __shfl_up_sync(0xffffffffu, ti, 1);
-        double trr = __shfl_down_sync(0xffffffffu, tr, 1), tir = __shfl_down_sync(0xffffffffu, ti, 1);
-        if (lane == 0) { trl = 0.0; til = 0.0; }
-        if (lane + 1 >= m) { trr = 0.0; tir = 0.0; }
-        double xr = fma(dk, tr, fma(ek, trl, fk * trr));
-        double xi = fma(dk, ti, fma(ek, til, fk * tir));
-        double nr, ni;
-        if (n == 0) { nr = xr; ni = xi; }
-        else { nr = fma(2.0, xr, -tmr); ni = fma(2.0, xi, -tmi); }
-        if (!on) { nr = 0.0; ni = 0.0; }
-        tmr = tr; tmi = ti;
-        tr = nr; ti = ni;
-      }
-      vre = accr;
-      vim = acci;
-    }
-  }
-  // global phase exp(-i s c)
-  double sn, cs;
-  sincos(-s * c, &sn, &cs);
-  const double rr = vre * cs - vim * sn;
-  const double ri = vre * sn + vim * cs;
-  if (on) { ure[lane] = rr; uim[lane] = ri; }
-}
-
 // Sum of nval doubles over the team, in a fixed order, identical on every CTA.  `mine`
-// holds this CTA's partials in shared memory and `out` receives the sums (shared memory).
+// holds this CTA's partials in shared memory; store(k, sum) runs on one thread of every CTA.
 // Cluster teams read the other CTAs' partials through distributed shared memory: callers
 // alternate between two `mine` buffers, so that one cluster barrier per call suffices (a
 // buffer is rewritten only after the next call's barrier, which every reader has passed).
 // Grid teams go through the global partial buffers.
-__device__ void team_reduce_vec(Team& tm, const double* mine, double* out, int nval) {
+template <typename F>
+__device__ __forceinline__ void team_reduce_vec(Team& tm, const double* mine, int nval, F&& store) {
   __syncthreads();
   if (tm.kind == TEAM_CLUSTER) {
     cg::cluster_group cl = cg::this_cluster();
-    cl.sync();
+    if (tm.size > 1) cl.sync();
     for (int k = threadIdx.x; k < nval; k += NT) {
       // the 16 peers' values loaded together, then added in a fixed tree (depth 4)
       double a[16];
@@ -698,7 +614,7 @@ __device__ void team_reduce_vec(Team& tm, const double* mine, double* out, int n
       for (int w = 8; w >= 1; w >>= 1)
 #pragma unroll
         for (int r = 0; r < w; ++r) a[r] += a[r + w];
-      out[k] = a[0];
+      store(k, a[0]);
     }
   } else {
     // grid team: each cluster first sums its CTAs' partials through distributed shared memory
@@ -726,393 +642,17 @@ __device__ void team_reduce_vec(Team& tm, const double* mine, double* out, int n
     for (int k = threadIdx.x; k < nval; k += NT) {
       double s = 0.0;
       for (int c = 0; c < ncl; ++c) s += buf[(long long)c * nval + k];
-      out[k] = s;
+      store(k, s);
     }
     tm.parity ^= 1;
   }
   __syncthreads();
 }
-
-// Butterfly sum of NV values over a warp (every lane ends with a full sum; lane 0's is used).
-// ------------------------------------------------------------------ Lanczos exponential
-struct KrylovShared {
-  double alpha[TTNS_KMAX + 1];
-  double beta[TTNS_KMAX + 2];   // beta[j] couples j-1 and j
-  double scale[TTNS_KMAX + 1];  // q_j = scale[j] * K_j
-  double ure[TTNS_KMAX];
-  double uim[TTNS_KMAX];
-  double rv[2][2 * (TTNS_KMAX + 1)];  // reorthogonalisation: per-CTA dot partials (alternating)
-  double rvo[2 * (TTNS_KMAX + 1)];    // and their team sums
-  int flag;
-};
-__shared__ KrylovShared s_ks;
-
-// Full reorthogonalisation of the FP64 path (the oracle's Lanczos does the same): two
-// classical Gram-Schmidt passes of w = K_{j+1} against q_i = scale_i K_i, i = 0..j,
-//   w <- w - sum_i <q_i, w> q_i,  <q_i, w> = scale_i <K_i, w>.
-// The dots are team sums (fixed order); each pass costs one team reduction.  The
-// functions return this thread's share of |w|^2 after the second pass.
-//
-// Vectors in global memory, elements idx = gtid + k * nthr (op_expm):
-__device__ double reorth_strided(Team& tm, long long N, const double2* x, const double2* Kb, long long kv,
-                                 double2* W, int j, KrylovShared& ks) {
-  __shared__ double s_wp[NWARP][16];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto Kp = [&](int i) -> const double2* { return i == 0 ? x : Kb + (long long)(i - 1) * kv; };
-  double nrm = 0.0;
-  for (int pass = 0; pass < 2; ++pass) {
-    double* mine = ks.rv[pass];
-    for (int i0 = 0; i0 <= j; i0 += 8) {
-      const int ni = min(8, j + 1 - i0);
-      double acc[16];
-#pragma unroll
-      for (int q = 0; q < 16; ++q) acc[q] = 0.0;
-      for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
-        const double2 w = W[idx];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          if (q < ni) {
-            const double2 k = Kp(i0 + q)[idx];
-            acc[2 * q] = fma(k.x, w.x, fma(k.y, w.y, acc[2 * q]));
-            acc[2 * q + 1] = fma(k.x, w.y, fma(-k.y, w.x, acc[2 * q + 1]));
-          }
-        }
-      }
-      warp_sum_n<16>(acc);
-      if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < 16; ++q) s_wp[warp][q] = acc[q];
-      __syncthreads();
-      if (threadIdx.x < 2 * ni) {
-        double sum = 0.0;
-        for (int w = 0; w < NWARP; ++w) sum += s_wp[w][threadIdx.x];
-        mine[2 * i0 + threadIdx.x] = sum;
-      }
-      __syncthreads();
-    }
-    team_reduce_vec(tm, mine, ks.rvo, 2 * (j + 1));
-    nrm = 0.0;
-    for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
-      double2 w = W[idx];
-      for (int i = 0; i <= j; ++i) {
-        const double sc = ks.scale[i];
-        const double cr = sc * ks.rvo[2 * i], ci = sc * ks.rvo[2 * i + 1];  // <q_i, w>
-        const double2 k0 = Kp(i)[idx];
-        const double2 k = make_double2(sc * k0.x, sc * k0.y);             // q_i
-        w.x -= cr * k.x - ci * k.y;
-        w.y -= cr * k.y + ci * k.x;
-      }
-      W[idx] = w;
-      nrm = fma(w.x, w.x, fma(w.y, w.y, nrm));
-    }
-  }
-  return nrm;
+__device__ void team_reduce_vec(Team& tm, const double* mine, double* out, int nval) {
+  team_reduce_vec(tm, mine, nval, [&](int k, double v) { out[k] = v; });
 }
 
-// Slices in shared memory, elements [0, n_own) of every K_i slice (op_expm_cluster):
-__device__ double reorth_slices(Team& tm, const double2* basis, long long S, int n_own, int j, KrylovShared& ks) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const double2* Kj1 = basis + (long long)(j + 1) * S;
-  double2* W = const_cast<double2*>(Kj1);
-  double nrm = 0.0;
-  for (int pass = 0; pass < 2; ++pass) {
-    double* mine = ks.rv[pass];
-    __syncthreads();  // w was written with the thread-strided mapping; the dots read it per lane
-    for (int i = warp; i <= j; i += NWARP) {  // warp per basis vector, lanes over the slice
-      const double2* Ki = basis + (long long)i * S;
-      double acc[2] = {0.0, 0.0};
-      for (int e = lane; e < n_own; e += 32) {
-        const double2 k = Ki[e], w = W[e];
-        acc[0] = fma(k.x, w.x, fma(k.y, w.y, acc[0]));
-        acc[1] = fma(k.x, w.y, fma(-k.y, w.x, acc[1]));
-      }
-      warp_sum_n<2>(acc);
-      if (lane == 0) {
-        mine[2 * i] = acc[0];
-        mine[2 * i + 1] = acc[1];
-      }
-    }
-    team_reduce_vec(tm, mine, ks.rvo, 2 * (j + 1));
-    nrm = 0.0;
-    for (int e = threadIdx.x; e < n_own; e += NT) {
-      double2 w = W[e];
-      for (int i = 0; i <= j; ++i) {
-        const double sc = ks.scale[i];
-        const double cr = sc * ks.rvo[2 * i], ci = sc * ks.rvo[2 * i + 1];  // <q_i, w>
-        const double2 k0 = basis[(long long)i * S + e];
-        const double2 k = make_double2(sc * k0.x, sc * k0.y);             // q_i
-        w.x -= cr * k.x - ci * k.y;
-        w.y -= cr * k.y + ci * k.x;
-      }
-      W[e] = w;
-      nrm = fma(w.x, w.x, fma(w.y, w.y, nrm));
-    }
-  }
-  return nrm;
-}
-
-
-struct PhaseClock {
-  long long t;
-  bool on;
-  bool grid;  // phases of grid-team ops go to their own counters
-  __device__ void start(bool enable, bool grid_team = false) {
-    on = enable;
-    grid = grid_team;
-    t = clock64();
-  }
-  __device__ void lap(Ctl* ctl, int phase) {
-    if (!on) return;
-    const long long now = clock64();
-    atomicAdd(grid ? &ctl->phase_cycles_grid[phase] : &ctl->phase_cycles[phase], (unsigned long long)(now - t));
-    t = now;
-  }
-};
-
-// Cluster-resident Krylov exponential for small nodes.  Each CTA of the cluster owns a
-// contiguous slice of every Krylov vector in its shared memory; the full input vector of
-// each application is all-gathered through distributed shared memory, every operator is
-// staged once, and the only global traffic is the node tensor in and out.  The arithmetic
-// is the same as op_expm's (same recurrence, same reductions, same convergence and
-// substep rules).
-template <typename T>
-__device__ __noinline__ bool op_expm_cluster(const KernelParams& P, Team& tm, const Instr& I, double tau) {
-  using V = typename C2<T>::t;
-  KrylovShared& ks = s_ks;
-  OpStage& os = s_os;
-  PhaseClock pc;
-  pc.start(P.profile && tm.rank == 0 && threadIdx.x == 0);
-  const NodeDesc nd = P.nodes[I.node];
-  const TermList L = P.lists[I.terms];
-  const long long N = nd.size;
-  const int cs = tm.size;
-  const long long S = (N + cs - 1) / cs;           // slice length
-  const long long e0 = (long long)tm.rank * S;
-  const long long e1 = min(N, e0 + S);
-  const int mmax = min(P.mmax, (int)(N < (long long)TTNS_KMAX ? N : (long long)TTNS_KMAX));
-  // shared-memory layout after the matrices: [xs: N V][tmp: n2*N V][basis: (mmax+1)*S double2]
-  {
-    const long long mats = (long long)(I.rega_len + I.regb_len) * sizeof(V);
-    long long off = (long long)(N + (long long)L.n2 * N) * sizeof(V);
-    off = (off + 15) & ~15LL;
-    const long long need = mats + 32 + off + (long long)(mmax + 1) * S * sizeof(double2) + S * (long long)sizeof(V);
-    if (need > P.smem_bytes) return false;  // same decision on every CTA (same sizes)
-  }
-  stage_op<T>(P, I, L, nullptr, 0, os);
-  unsigned char* base = dyn_smem + ((long long)os.end * sizeof(double2));
-  V* xs = reinterpret_cast<V*>(base);
-  V* tmp = xs + N;
-  long long off = (long long)(N + (long long)L.n2 * N) * sizeof(V);
-  off = (off + 15) & ~15LL;
-  double2* basis = reinterpret_cast<double2*>(base + off);
-  // mixed precision: the own slice of the current Krylov vector in the compute type, which
-  // the other CTAs gather (converted once, by its owner)
-  constexpr bool kShadow = !std::is_same<T, double>::value;
-  V* kf = reinterpret_cast<V*>(basis + (long long)(mmax + 1) * S);
-  cg::cluster_group cl = cg::this_cluster();
-  auto Ks = [&](int j) -> double2* { return basis + (long long)j * S; };
-  double2* x = P.pool + nd.off;
-  double s_rem = I.sign * tau / HBAR_EVFS;
-  int total_m = 0, m = 0;
-  for (long long e = e0 + threadIdx.x; e < e1; e += NT) Ks(0)[e - e0] = x[e];
-  __syncthreads();
-  pc.lap(P.ctl, 0);
-  for (int chunk = 0; chunk < 64; ++chunk) {
-    double v[1] = {0.0};
-    for (long long e = e0 + threadIdx.x; e < e1; e += NT) {
-      const double2 a = Ks(0)[e - e0];
-      v[0] = fma(a.x, a.x, fma(a.y, a.y, v[0]));
-      if constexpr (kShadow) kf[e - e0] = cvt<T>(a);
-    }
-    team_allreduce(tm, v, 1);
-    const double beta0 = sqrt(v[0]);
-    pc.lap(P.ctl, 6);
-    if (!(beta0 > 0.0)) {
-      if (!(beta0 == 0.0)) set_status(P.ctl, ST_NONFINITE, I.op, I.node);
-      break;
-    }
-    if (threadIdx.x == 0) {
-      ks.scale[0] = 1.0 / beta0;
-      ks.beta[0] = 0.0;
-    }
-    __syncthreads();
-    m = 0;
-    bool conv = false;
-    double bnext = 0.0, lead = 1.0;
-    int next_check = 1;
-    for (int j = 0; j < mmax; ++j) {
-      // all-gather K_j (complete on every CTA: written before the last cluster barrier),
-      // from the compute-type slices in mixed precision
-      {
-        V* src = kShadow ? kf : reinterpret_cast<V*>(Ks(j));
-        const float invS = 1.0f / (float)S;
-        int e = threadIdx.x;
-        for (; e + 3 * NT < (int)N; e += 4 * NT) {
-          V a[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int ee = e + q * NT;
-            const int r = fdivu(ee, (int)S, invS);
-            a[q] = cl.map_shared_rank(src, r)[ee - r * (int)S];
-          }
-#pragma unroll
-          for (int q = 0; q < 4; ++q) xs[e + q * NT] = a[q];
-        }
-        for (; e < (int)N; e += NT) {
-          const int r = fdivu(e, (int)S, invS);
-          xs[e] = cl.map_shared_rank(src, r)[e - r * (int)S];
-        }
-      }
-      __syncthreads();
-      if (L.n2 > 0) {
-        // first factors of the two-stage terms, on the elements that the own slice's second
-        // factors read: the slice widened to whole blocks of the second factor's leg (every
-        // CTA computes its range from the gathered input; for a factor on the last leg the
-        // range is the slice's rows)
-        const int t0 = L.count - L.n2;
-        for (int t = 0; t < L.n2; ++t) {
-          const int l2 = os.terms[t0 + t].f[1].leg;
-          const long long blk = (long long)nd.dims[l2] * nd.strides[l2];
-          const long long lo = e1 > e0 ? (e0 / blk) * blk : 0;
-          const long long hi = e1 > e0 ? min(N, ((e1 - 1) / blk + 1) * blk) : 0;
-          for (long long e = lo + threadIdx.x; e < hi; e += NT)
-            tmp[t * N + e] = factor_dot<T>(P, nd, os.terms[t0 + t].f[0], os, xs, e);
-        }
-        __syncthreads();
-      }
-      pc.lap(P.ctl, 1);
-      const double sj = ks.scale[j], bj = ks.beta[j];
-      const double sjm = j > 0 ? ks.scale[j - 1] : 0.0;
-      double2* W = Ks(j + 1);
-      // part[0] = Re <K_j, w>; in mixed precision also part[1] = |w|^2, so that one team
-      // reduction gives both alpha_j and beta_{j+1}
-      const bool mixed = P.precision != 0;
-      double part[3] = {0.0, 0.0, 0.0};
-      for (long long e = e0 + threadIdx.x; e < e1; e += NT) {
-        const auto a = apply_stage2_at<T>(P, nd, xs, L, tmp, N, e, os);
-        const double2 kj = Ks(j)[e - e0];
-        double wr = sj * (double)a.x, wi = sj * (double)a.y;
-        if (j > 0) {
-          const double2 km = Ks(j - 1)[e - e0];
-          wr = fma(-bj * sjm, km.x, wr);
-          wi = fma(-bj * sjm, km.y, wi);
-        }
-        W[e - e0] = make_double2(wr, wi);
-        part[0] = fma(kj.x, wr, fma(kj.y, wi, part[0]));
-        if (mixed) {
-          part[1] = fma(wr, wr, fma(wi, wi, part[1]));
-          part[2] = fma(kj.x, kj.x, fma(kj.y, kj.y, part[2]));
-        }
-      }
-      team_allreduce(tm, part, mixed ? 3 : 1);
-      pc.lap(P.ctl, 2);
-      const double aj = part[0] * sj;
-      // |w - alpha_j q_j|^2 = |w|^2 - 2 alpha_j^2 + alpha_j^2 |q_j|^2 with |q_j|^2 from the same
-      // reduction (the error of an assumed |q_j| = 1 would grow by alpha^2 / beta^2 per step);
-      // used unless it cancels (the same decision on every CTA)
-      const double nq = sj * sj * part[2];
-      const double b2 = part[1] - aj * aj * (2.0 - nq);
-      const bool fused = mixed && b2 > 1e-4 * part[1];
-      double nrm[1] = {0.0};
-      for (long long e = e0 + threadIdx.x; e < e1; e += NT) {
-        const double2 kj = Ks(j)[e - e0];
-        double2 w = W[e - e0];
-        w.x = fma(-aj * sj, kj.x, w.x);
-        w.y = fma(-aj * sj, kj.y, w.y);
-        W[e - e0] = w;
-        if constexpr (kShadow) kf[e - e0] = cvt<T>(w);  // gathered after the next barrier
-        nrm[0] = fma(w.x, w.x, fma(w.y, w.y, nrm[0]));
-      }
-      if (P.precision == 0) nrm[0] = reorth_slices(tm, basis, S, (int)max(0LL, e1 - e0), j, ks);
-      if (fused) {
-        bnext = sqrt(b2);
-        cl.sync();  // the slices of K_{j+1} are complete before any CTA gathers them
-      } else {
-        team_allreduce(tm, nrm, 1);
-        bnext = sqrt(nrm[0]);
-      }
-      pc.lap(P.ctl, 3);
-      if (threadIdx.x == 0) {
-        ks.alpha[j] = aj;
-        ks.beta[j + 1] = bnext;
-        ks.scale[j + 1] = bnext > 0.0 ? 1.0 / bnext : 0.0;
-      }
-      __syncthreads();
-      m = j + 1;
-      const double est = bnext * lead;
-      lead *= fabs(s_rem) * bnext / (double)m;
-      if ((est <= 1e2 * P.tol && m >= next_check) || m == mmax || !(bnext > 0.0)) {
-        next_check = m + 1;
-        if (threadIdx.x < 32) texp_warp(ks.alpha, ks.beta, m, s_rem, ks.ure, ks.uim);
-        __syncthreads();
-        const double um = sqrt(ks.ure[m - 1] * ks.ure[m - 1] + ks.uim[m - 1] * ks.uim[m - 1]);
-        const double err = bnext * um;
-        if (!(err == err)) {
-          set_status(P.ctl, ST_NONFINITE, I.op, I.node);
-          conv = true;
-        } else if (err <= P.tol || !(bnext > 0.0)) {
-          conv = true;
-        }
-        pc.lap(P.ctl, 4);
-        if (conv || m == mmax) break;
-      }
-    }
-    total_m += m;
-    double s_done = s_rem;
-    if (!conv && m < N) {
-      for (int k = 0; k < 30; ++k) {
-        s_done *= 0.5;
-        if (threadIdx.x < 32) texp_warp(ks.alpha, ks.beta, m, s_done, ks.ure, ks.uim);
-        __syncthreads();
-        const double um = sqrt(ks.ure[m - 1] * ks.ure[m - 1] + ks.uim[m - 1] * ks.uim[m - 1]);
-        __syncthreads();
-        if (bnext * um <= P.tol) break;
-      }
-      pc.lap(P.ctl, 4);
-    }
-    // y = beta0 sum_k u_k q_k into the own slice of K_0
-    double ny[1] = {0.0};
-    for (long long e = e0 + threadIdx.x; e < e1; e += NT) {
-      double yr = 0.0, yi = 0.0;
-      for (int k = 0; k < m; ++k) {
-        const double2 q = Ks(k)[e - e0];
-        const double sc = beta0 * ks.scale[k];
-        const double cr = ks.ure[k] * sc, ci = ks.uim[k] * sc;
-        yr = fma(cr, q.x, fma(-ci, q.y, yr));
-        yi = fma(cr, q.y, fma(ci, q.x, yi));
-      }
-      Ks(0)[e - e0] = make_double2(yr, yi);
-      ny[0] = fma(yr, yr, fma(yi, yi, ny[0]));
-    }
-    if (P.precision != 0) {
-      team_allreduce(tm, ny, 1);
-      const double ratio = ny[0] > 0.0 ? beta0 / sqrt(ny[0]) : 1.0;
-      if (fabs(ratio - 1.0) < 1e-3)
-        for (long long e = e0 + threadIdx.x; e < e1; e += NT) {
-          const double2 y = Ks(0)[e - e0];
-          Ks(0)[e - e0] = make_double2(y.x * ratio, y.y * ratio);
-        }
-    }
-    __syncthreads();
-    pc.lap(P.ctl, 5);
-    if (conv || m >= N || s_done == s_rem) break;
-    s_rem -= s_done;
-    if (chunk == 63 && tm.rank == 0 && threadIdx.x == 0) {
-      // 64 Krylov spaces did not cover the time step: the result is incomplete
-      atomicAdd(&P.ctl->not_converged, 1ull);
-      set_status(P.ctl, ST_NOT_CONVERGED, I.op, I.node);
-    }
-  }
-  for (long long e = e0 + threadIdx.x; e < e1; e += NT) x[e] = Ks(0)[e - e0];
-  if (tm.rank == 0 && threadIdx.x == 0) {
-    P.mhist[I.hist] = m;
-    atomicAdd(&P.ctl->krylov_iters, (unsigned long long)total_m);
-    atomicAdd(&P.ctl->applies, (unsigned long long)total_m);
-    atomicAdd(&P.ctl->flops, I.flops * total_m);
-  }
-  team_sync(tm);
-  return true;
-}
+#include "krylov.cuh"
 
 // Tiled apply for grid-team nodes too large for shared memory.  The node (legs 0..nl-1, the
 // last one physical) is covered twice by tiles:
@@ -1784,34 +1324,24 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
     for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
       const double2 a = x[idx];
       v[0] = fma(a.x, a.x, fma(a.y, a.y, v[0]));
-      if (shadow) xf[idx] = cvt<T>(a);
+      if constexpr (kShadow) xf[idx] = cvt<T>(a);
     }
-    team_allreduce(tm, v, 1);
-    const double beta0 = sqrt(v[0]);
+    team_reduce<1>(tm, v, [&](const double* t) { krylov_begin(ks, t[0]); });
     pc.lap(P.ctl, 6);
+    const double beta0 = ks.beta0;
     if (!(beta0 > 0.0)) {
       if (!(beta0 == 0.0)) set_status(P.ctl, ST_NONFINITE, I.op, I.node);
       break;
     }
-    if (threadIdx.x == 0) {
-      ks.scale[0] = 1.0 / beta0;
-      ks.beta[0] = 0.0;
-    }
-    __syncthreads();
     m = 0;
     bool conv = false;
-    double bnext = 0.0;
-    // leading-order size of |e_m^T exp(-i s T_m) e_0|: |s|^(m-1) prod beta_i / (m-1)!,
-    // used to decide when the exact (small-exponential) check is worth running
-    double lead = 1.0;
-    int next_check = 1;
+    double nsq = v[0];  // this thread's share of |K_j|^2
     for (int j = 0; j < mmax; ++j) {
       double2* Kj = Kp(j);
       double2* Kjm = j > 0 ? Kp(j - 1) : x;
       double2* W = Kb + (long long)j * kv;  // slot of K_{j+1}
       const double sj = ks.scale[j];
-      const double bj = ks.beta[j];
-      const double sjm = j > 0 ? ks.scale[j - 1] : 0.0;
+      const double cm = ks.cm;  // beta_j scale_{j-1}
       if (xs) {
         if constexpr (kShadow)
           stage_copy(xs, xf, N);
@@ -1825,24 +1355,21 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
         team_sync(tm);
       }
       pc.lap(P.ctl, 1);
-      // part[0] = Re <K_j, w>; in mixed precision also part[1] = |w|^2 (one reduction for
-      // alpha_j and beta_{j+1}, as in the cluster-resident form)
-      const bool mixed = P.precision != 0;
-      double part[3] = {0.0, 0.0, 0.0};
-      auto recur = [&](long long idx, V a) {  // w = s_j H K_j - beta_j q_{j-1} at idx, and the dots
+      // part[0] = Re <K_j, w>; in mixed precision also part[1] = |w|^2 and part[2] = |K_j|^2
+      // (one reduction for alpha_j and beta_{j+1}, as in the cluster-resident form)
+      double part[3] = {0.0, 0.0, nsq};
+      // w = s_j H K_j - beta_j q_{j-1} at idx, and the dots
+      auto recur = [&](long long idx, V a) {
+        double wr = sj * to_f64(a.x), wi = sj * to_f64(a.y);
         const double2 kj = Kj[idx];
-        double wr = sj * (double)a.x, wi = sj * (double)a.y;
         if (j > 0) {
           const double2 km = Kjm[idx];
-          wr = fma(-bj * sjm, km.x, wr);
-          wi = fma(-bj * sjm, km.y, wi);
+          wr = fma(-cm, km.x, wr);
+          wi = fma(-cm, km.y, wi);
         }
-        W[idx] = make_double2(wr, wi);
         part[0] = fma(kj.x, wr, fma(kj.y, wi, part[0]));  // Re(conj(K_j) w)
-        if (mixed) {
-          part[1] = fma(wr, wr, fma(wi, wi, part[1]));
-          part[2] = fma(kj.x, kj.x, fma(kj.y, kj.y, part[2]));
-        }
+        if constexpr (kShadow) part[1] = fma(wr, wr, fma(wi, wi, part[1]));
+        W[idx] = make_double2(wr, wi);
       };
       if (use_tc) {
         tc_apply<T>(P, tm, nd, os, s_tcp, xin, ybuf, kv);
@@ -1863,92 +1390,69 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
       } else {
         for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) recur(idx, apply_stage2_at<T>(P, nd, xin, L, tmp, kv, idx, os));
       }
-      team_allreduce(tm, part, mixed ? 3 : 1);
+      if constexpr (kShadow)
+        team_reduce<3>(tm, part, [&](const double* t) { krylov_alpha(ks, j, t[0], t[1], t[2]); });
+      else
+        team_reduce<1>(tm, part, [&](const double* t) { krylov_alpha(ks, j, t[0]); });
       pc.lap(P.ctl, 2);
-      const double aj = part[0] * sj;
-      // |w - alpha_j q_j|^2 = |w|^2 - 2 alpha_j^2 + alpha_j^2 |q_j|^2 with |q_j|^2 from the same
-      // reduction (the error of an assumed |q_j| = 1 would grow by alpha^2 / beta^2 per step);
-      // used unless it cancels (the same decision on every CTA)
-      const double nq = sj * sj * part[2];
-      const double b2 = part[1] - aj * aj * (2.0 - nq);
-      const bool fused = mixed && b2 > 1e-4 * part[1];
+      const double ca = ks.ca;  // alpha_j scale_j
+      if (kShadow && ks.fused && threadIdx.x == NT - 32) krylov_norm(ks, j, ks.b2, s_rem, P.tol, mmax);
       double nrm[1] = {0.0};
       for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
         const double2 kj = Kj[idx];
         double2 w = W[idx];
-        w.x = fma(-aj * sj, kj.x, w.x);
-        w.y = fma(-aj * sj, kj.y, w.y);
+        w.x = fma(-ca, kj.x, w.x);
+        w.y = fma(-ca, kj.y, w.y);
         W[idx] = w;
-        if (shadow) xf[idx] = cvt<T>(w);  // every read of the old shadow ended at the last barrier
-        nrm[0] = fma(w.x, w.x, fma(w.y, w.y, nrm[0]));
-      }
-      if (P.precision == 0) nrm[0] = reorth_strided(tm, N, x, Kb, kv, W, j, ks);
-      if (fused) {
-        bnext = sqrt(b2);
-        team_sync(tm);  // K_{j+1} and its shadow are complete before the next application
-      } else {
-        team_allreduce(tm, nrm, 1);
-        bnext = sqrt(nrm[0]);
-      }
-      pc.lap(P.ctl, 3);
-      if (threadIdx.x == 0) {
-        ks.alpha[j] = aj;
-        ks.beta[j + 1] = bnext;
-        ks.scale[j + 1] = bnext > 0.0 ? 1.0 / bnext : 0.0;
-      }
-      __syncthreads();
-      m = j + 1;
-      const double est = bnext * lead;
-      lead *= fabs(s_rem) * bnext / (double)m;
-      if ((est <= 1e2 * P.tol && m >= next_check) || m == mmax || !(bnext > 0.0)) {
-        next_check = m + 1;
-        if (threadIdx.x < 32) texp_warp(ks.alpha, ks.beta, m, s_rem, ks.ure, ks.uim);
-        __syncthreads();
-        const double um = sqrt(ks.ure[m - 1] * ks.ure[m - 1] + ks.uim[m - 1] * ks.uim[m - 1]);
-        const double err = bnext * um;
-        if (!(err == err)) {
-          set_status(P.ctl, ST_NONFINITE, I.op, I.node);
-          conv = true;
-        } else if (err <= P.tol || !(bnext > 0.0)) {
-          conv = true;
+        if constexpr (kShadow) {
+          xf[idx] = cvt<T>(w);  // every read of the old shadow ended at the last barrier
+          nrm[0] = fma(w.x, w.x, fma(w.y, w.y, nrm[0]));
         }
+      }
+      if constexpr (!kShadow) {
+        nrm[0] = orth_strided(tm, N, x, Kb, kv, W, j, ks);
+        if (ks.fused && threadIdx.x == NT - 32) krylov_norm(ks, j, ks.b2, s_rem, P.tol, mmax);
+      }
+      const bool fused = ks.fused != 0;
+      nsq = nrm[0];
+      if (fused)
+        team_sync(tm);  // K_{j+1} and its shadow are complete before the next application
+      else
+        team_reduce<1>(tm, nrm, [&](const double* t) { krylov_norm(ks, j, t[0], s_rem, P.tol, mmax); });
+      pc.lap(P.ctl, 3);
+      m = j + 1;
+      if (ks.check) {
+        if (threadIdx.x < 32) krylov_check(ks, m, s_rem, P.tol);
+        __syncthreads();
+        conv = ks.conv != 0;
+        if (ks.conv == 2) set_status(P.ctl, ST_NONFINITE, I.op, I.node);
         pc.lap(P.ctl, 4);
         if (conv || m == mmax) break;
       }
     }
     total_m += m;
-    double s_done = s_rem;
-    if (!conv && m < N) {
-      // largest s_rem / 2^k that converges on this space (same decision on every CTA)
-      for (int k = 0; k < 30; ++k) {
-        s_done *= 0.5;
-        if (threadIdx.x < 32) texp_warp(ks.alpha, ks.beta, m, s_done, ks.ure, ks.uim);
-        __syncthreads();
-        const double um = sqrt(ks.ure[m - 1] * ks.ure[m - 1] + ks.uim[m - 1] * ks.uim[m - 1]);
-        __syncthreads();
-        if (bnext * um <= P.tol) break;
-      }
-      pc.lap(P.ctl, 4);
-    }
+    if (threadIdx.x < 32) krylov_exp(ks, m, s_rem, P.tol, !conv && m < N);
+    __syncthreads();
+    const double s_done = ks.s_done;
+    pc.lap(P.ctl, 4);
     // y = beta0 * sum_k u_k q_k written over x (each thread reads its own K_0 = x entries first)
     double ny[1] = {0.0};
     for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
       double yr = 0.0, yi = 0.0;
       for (int k = 0; k < m; ++k) {
         const double2 q = Kp(k)[idx];
-        const double sc = beta0 * ks.scale[k];
-        const double cr = ks.ure[k] * sc, ci = ks.uim[k] * sc;
+        const double cr = ks.ure[k], ci = ks.uim[k];
         yr = fma(cr, q.x, fma(-ci, q.y, yr));
         yi = fma(cr, q.y, fma(ci, q.x, yi));
       }
       x[idx] = make_double2(yr, yi);
       ny[0] = fma(yr, yr, fma(yi, yi, ny[0]));
     }
-    if (P.precision != 0) {
+    if constexpr (kShadow) {
       // The exact exponential is unitary.  FP32-class contractions leave the Krylov basis
       // orthonormal only to ~1e-7, so the combination's norm is restored to the input's.
-      team_allreduce(tm, ny, 1);
-      const double ratio = ny[0] > 0.0 ? beta0 / sqrt(ny[0]) : 1.0;
+      team_reduce<1>(tm, ny, [&](const double* t) { ks.ratio = t[0] > 0.0 ? ks.beta0 / sqrt(t[0]) : 1.0; });
+      const double ratio = ks.ratio;
       if (fabs(ratio - 1.0) < 1e-3) {
         for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
           double2 y = x[idx];
@@ -2581,7 +2085,7 @@ __device__ void exec_op(const KernelParams& P, Team& tm, const Instr& I, double2
   switch (I.op) {
     case OP_FWD:
     case OP_BOND:
-      if (!(tm.kind == TEAM_CLUSTER && P.cluster_resident && op_expm_cluster<T>(P, tm, I, tau)))
+      if (!(tm.kind == TEAM_CLUSTER && P.cluster_resident && op_expm_cluster<T>(P, tm, I, work, tau)))
         op_expm<T>(P, tm, I, work, tau);
       break;
     case OP_QR:
