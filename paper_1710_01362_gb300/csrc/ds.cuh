@@ -96,13 +96,7 @@ struct DsAcc {
   __device__ __forceinline__ float2 val() const { return ds_quick(s, c); }
 };
 
-// complex accumulators: (ar, ai) += conj(v) w, and (ar, ai) += a b
-__device__ __forceinline__ void ds_conj_mac(DsAcc& ar, DsAcc& ai, float4 v, float4 w) {
-  ar.mac(ds_re(v), ds_re(w));
-  ar.mac(ds_im(v), ds_im(w));
-  ai.mac(ds_re(v), ds_im(w));
-  ai.mac(ds_neg(ds_im(v)), ds_re(w));
-}
+// complex accumulators: (ar, ai) += a b
 __device__ __forceinline__ void ds_cmac(DsAcc& ar, DsAcc& ai, float4 a, float4 b) {
   ar.mac(ds_re(a), ds_re(b));
   ar.mac(ds_neg(ds_im(a)), ds_im(b));
@@ -112,28 +106,6 @@ __device__ __forceinline__ void ds_cmac(DsAcc& ar, DsAcc& ai, float4 a, float4 b
 
 __device__ __forceinline__ float2 shfl_xor_ds(float2 v, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
-}
-
-// warp_reduce_t for double-single values: lane L returns the total of value
-// warp_reduce_vid<V>(L)
-template <int V>
-__device__ __forceinline__ float2 warp_reduce_ds_t(float2* v) {
-  const int lane = threadIdx.x & 31;
-  int off = 16;
-#pragma unroll
-  for (int n = V; n > 1; n >>= 1, off >>= 1) {
-    const bool hi = (lane & off) != 0;
-#pragma unroll
-    for (int i = 0; i < n / 2; ++i) {
-      const float2 send = hi ? v[i] : v[i + n / 2];
-      const float2 keep = hi ? v[i + n / 2] : v[i];
-      v[i] = ds_add(keep, shfl_xor_ds(send, off));
-    }
-  }
-  float2 t = v[0];
-#pragma unroll
-  for (; off > 0; off >>= 1) t = ds_add(t, shfl_xor_ds(t, off));
-  return t;
 }
 
 }  // namespace ttns

@@ -1478,415 +1478,7 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
   }
 }
 
-// ------------------------------------------------------------------ Householder QR
-// A_v (matricised: rows = all other legs in order, columns = leg I.leg) = Q R with the
-// completion rule of the oracle: null sub-columns (norm <= qr_cutoff ||M||_F) get the identity
-// reflector and R_jj = 0; Q = H_0 ... H_{n-1} I[:, :n] through the compact WY form
-// Q = I - V T V^H; finally R_jj is made real and >= 0.  FP64.
-struct QRShared {
-  double tau[TTNS_MAX_D];    // H_j = I - tau_j v_j v_j^H with the unnormalised v_j of the column loop
-  double shat[TTNS_MAX_D];   // 1 / |v_j| = sqrt(tau_j / 2) (0 for an identity reflector)
-  double2 coef[TTNS_MAX_D];  // tau_j v_j^H W[k] of the trailing columns
-  double2 vhead[TTNS_MAX_D];
-  double2 rdiag[TTNS_MAX_D];
-  double2 ph[TTNS_MAX_D];
-};
-__shared__ QRShared s_qs;
-
-
-__device__ __forceinline__ long long qr_addr(const NodeDesc& nd, int l, long long r, int c) {
-  const int st = nd.strides[l];
-  const int p = fdivu((int)r, st, nd.inv_strides[l]);
-  const int q = (int)r - p * st;
-  return (long long)(p * nd.dims[l] * st + c * st + q);
-}
-
-// Every CTA of the team owns a contiguous chunk of rows [rb, re); loops inside a CTA run
-// over (column, row) pairs so that small chunks (a few rows per CTA) still occupy the
-// threads.  The FP64 work is spread over all SMs of the team.
-__device__ __noinline__ void op_qr(const KernelParams& P, Team& tm, const Instr& I, double2* work) {
-  QRShared& qs = s_qs;
-  PhaseClock pc;
-  pc.start(P.profile && tm.rank == 0 && threadIdx.x == 0, tm.kind == TEAM_GRID);
-  const NodeDesc nd = P.nodes[I.node];
-  const int l = I.leg;
-  const int n = nd.dims[l];
-  const long long rows = nd.size / n;
-  double2* A = P.pool + nd.off;
-  double2* W = work;  // column-major: W[c * rows + r]
-  double2* Rout = P.pool + P.trees[I.tree].bond_off;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long chunk = (rows + tm.size - 1) / tm.size;
-  const long long rb = min(rows, (long long)tm.rank * chunk);
-  const long long re = min(rows, rb + chunk);
-  const int nr = (int)(re - rb);
-  const float inv_nr = nr > 0 ? 1.0f / (float)nr : 0.0f;
-  // reduction buffers in the dynamic shared memory (no operator is staged during a QR)
-  const int PB = max(2 * n * n, 4 * n + 4);
-  double* red[2] = {reinterpret_cast<double*>(dyn_smem), reinterpret_cast<double*>(dyn_smem) + PB};
-  double* redo = red[1] + PB;
-  int rp = 0;
-  // the CTA's own rows of the workspace matrix stay in shared memory during the QR when
-  // they fit (column-major, `chunk` rows per column); rows < n, which other CTAs read for T,
-  // Z and R, are also written to the global workspace after the column loop
-  const long long ws_off = (3LL * PB * (long long)sizeof(double) + 15) & ~15LL;
-  const bool in_smem = ws_off + (long long)n * chunk * (long long)sizeof(double2) <= P.smem_bytes;
-  double2* const Wl = in_smem ? reinterpret_cast<double2*>(dyn_smem + ws_off) : W;
-  const long long ldw = in_smem ? chunk : rows;
-  const long long roff = in_smem ? rb : 0;
-  auto WA = [&](int c, long long r) -> double2& { return Wl[(long long)c * ldw + (r - roff)]; };
-  // the small matrices G (Gram of the reflectors), T and Z (n x n, row stride ldg): after the
-  // rows in shared memory when they fit there too, else in the per-CTA global scratch
-  const long long g_off = (ws_off + (in_smem ? (long long)n * chunk * (long long)sizeof(double2) : 0) + 15) & ~15LL;
-  const bool g_smem = g_off + 3LL * n * n * (long long)sizeof(double2) <= P.smem_bytes;
-  const int ldg = g_smem ? n : TTNS_MAX_D;
-  double2* G = g_smem ? reinterpret_cast<double2*>(dyn_smem + g_off)
-                      : P.cta_scratch + (long long)blockIdx.x * P.cta_scratch_stride;
-  double2* Tm = G + ldg * ldg;
-  double2* Z = Tm + ldg * ldg;
-  // copy into the column-major workspace; the Frobenius norm sets the null threshold
-  double fro = 0.0;
-  for (int idx = threadIdx.x; idx < n * nr; idx += NT) {
-    const int c = fdivu(idx, nr, inv_nr);
-    const long long r = rb + (idx - c * nr);
-    const double2 a = A[qr_addr(nd, l, r, c)];
-    WA(c, r) = a;
-    fro = fma(a.x, a.x, fma(a.y, a.y, fro));
-  }
-  __syncthreads();  // copied with the pair mapping, read below per lane
-  // One team reduction per column.  Before reflecting column j every CTA needs, over its
-  // rows r > j and for the columns c = j .. n-1,
-  //   d_c = sum_r conj(W[j][r]) W[c][r]   and   h_c = W[c][j]  (row j: its owner only),
-  // in slots [4 (c - j) .. 4 (c - j) + 4).  Then sigma_j^2 = |h_j|^2 + d_j, x0 = h_j, and
-  // c_k = tau (d_k + conj(vh) h_k) is v^H W[k] with the head of v replaced by vh.
-  // Products and sums are packed so that few FP64 instructions run with idle lanes: when
-  // the CTA's rows below jj number at most 32, one thread forms each (column, row) product
-  // into shared memory and the per-column sums are fixed trees; for more rows, warps take
-  // columns four at a time with a transposing butterfly.
-  // product scratch (n x 32 complex) after G, T, Z
-  const long long p_off = (g_off + (g_smem ? 3LL * n * n * (long long)sizeof(double2) : 0) + 15) & ~15LL;
-  const bool p_smem = g_smem && p_off + 32LL * n * (long long)sizeof(double2) <= P.smem_bytes;
-  double2* const prod = reinterpret_cast<double2*>(dyn_smem + p_off);
-  auto prepare = [&](int jj, double* mine) {
-    const int nc = n - jj;
-    const long long r1 = max(rb, (long long)jj + 1);
-    const int nrw = (int)max(0LL, re - r1);  // own rows strictly below row jj
-    if (p_smem && chunk <= 32) {  // the same branch on every CTA (chunk is uniform)
-      // prod[c * 32 + r] = conj(v_r) W[jj + c][r], zero-padded to 32 rows
-      for (int idx = threadIdx.x; idx < nc * 32; idx += NT) {
-        const int c = idx >> 5, rr = idx & 31;
-        double2 p = make_double2(0.0, 0.0);
-        if (rr < nrw) {
-          const long long r = r1 + rr;
-          const double2 vr = WA(jj, r), w = WA(jj + c, r);
-          p = make_double2(fma(vr.x, w.x, vr.y * w.y), fma(vr.x, w.y, -vr.y * w.x));
-        }
-        prod[idx] = p;
-      }
-      __syncthreads();
-      // per column: 8 threads add 4 rows each, then a fixed tree over the 8 partials (the
-      // trip count is rounded to whole warps so that every lane takes part in the shuffles)
-      const int ntask = nc * 8;
-      for (int idx = threadIdx.x; idx < ((ntask + 31) & ~31); idx += NT) {
-        const bool on = idx < ntask;
-        const int c = idx >> 3, g = idx & 7;
-        double sr = 0.0, si = 0.0;
-        if (on) {
-          const double2* pc2 = prod + c * 32 + g;
-          const double2 s0 = pc2[0], s1 = pc2[8], s2 = pc2[16], s3 = pc2[24];
-          sr = (s0.x + s1.x) + (s2.x + s3.x);
-          si = (s0.y + s1.y) + (s2.y + s3.y);
-        }
-#pragma unroll
-        for (int o = 4; o >= 1; o >>= 1) {  // within the aligned group of 8 lanes
-          sr += __shfl_xor_sync(0xffffffffu, sr, o);
-          si += __shfl_xor_sync(0xffffffffu, si, o);
-        }
-        if (on && g == 0) {
-          mine[4 * c] = sr;
-          mine[4 * c + 1] = si;
-        }
-      }
-    } else {
-      for (int c0 = 0; c0 < nc; c0 += 4 * NWARP) {
-        double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (long long r = r1 + lane; r < re; r += 32) {
-          const double2 vr = WA(jj, r);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int c = c0 + warp + q * NWARP;
-            if (c < nc) {
-              const double2 w = WA(jj + c, r);
-              acc[2 * q] = fma(vr.x, w.x, fma(vr.y, w.y, acc[2 * q]));
-              acc[2 * q + 1] = fma(vr.x, w.y, fma(-vr.y, w.x, acc[2 * q + 1]));
-            }
-          }
-        }
-        const double t = warp_reduce_t<8>(acc);
-        if ((lane & 3) == 0) {
-          const int vid = warp_reduce_vid<8>(lane);
-          const int c = c0 + warp + (vid >> 1) * NWARP;
-          if (c < nc) mine[4 * c + (vid & 1)] = t;
-        }
-      }
-    }
-    const bool own_row = rb <= jj && jj < re;
-    for (int c = threadIdx.x; c < nc; c += NT) {
-      const double2 h = own_row ? WA(jj + c, jj) : make_double2(0.0, 0.0);
-      mine[4 * c + 2] = h.x;
-      mine[4 * c + 3] = h.y;
-    }
-  };
-  {
-    double* mine = red[rp];
-    rp ^= 1;
-    prepare(0, mine);
-    // the Frobenius norm rides along in the first reduction
-    __shared__ double s_fro[NWARP];
-    const double f = warp_sum(fro);
-    if (lane == 0) s_fro[warp] = f;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double sum = 0.0;
-      for (int w = 0; w < NWARP; ++w) sum += s_fro[w];
-      mine[4 * n] = sum;
-    }
-    team_reduce_vec(tm, mine, redo, 4 * n + 1);
-  }
-  pc.lap(P.ctl, 8);
-  const double fro_m = sqrt(redo[4 * n]);  // ||M||_F (redo is reused by the column loop)
-  const double thr = P.qr_cutoff * fro_m;
-  for (int j = 0; j < n; ++j) {
-    // reflector of column j: alpha = -phase(x0) sigma, vh = x0 - alpha = x0 (1 + sigma / |x0|),
-    // |vh| = |x0| + sigma, |v|^2 = d_j + |vh|^2, tau = 2 / |v|^2.  Written so that the FP64
-    // square roots and divisions (long dependent sequences on this part) overlap.
-    const double2 x0 = make_double2(redo[2], redo[3]);
-    const double ax2 = x0.x * x0.x + x0.y * x0.y;
-    const double sigma = sqrt(ax2 + redo[0]);
-    const double ax = sqrt(ax2);
-    double tau = 0.0, shat = 0.0;
-    double2 vh = make_double2(0, 0), alpha = make_double2(0, 0);
-    const bool null = !(sigma > thr);
-    if (!null) {
-      // a head below 1e-280 counts as zero (phase 1): its reciprocal would overflow
-      const bool head = ax > 1e-280;
-      const double inv_ax = head ? 1.0 / ax : 0.0;
-      const double hv = ax + sigma;
-      const double vn2 = redo[0] + hv * hv;
-      tau = 2.0 / vn2;
-      shat = rsqrt(vn2);
-      if (head) {
-        const double f = sigma * inv_ax;
-        alpha = make_double2(-f * x0.x, -f * x0.y);
-        vh = make_double2(x0.x + f * x0.x, x0.y + f * x0.y);
-      } else {
-        alpha = make_double2(-sigma, 0.0);
-        vh = make_double2(sigma, 0.0);
-      }
-    }
-    const int nk = n - j - 1;
-    if (threadIdx.x == 0) {
-      qs.tau[j] = tau;
-      qs.shat[j] = shat;
-      qs.vhead[j] = vh;
-      qs.rdiag[j] = alpha;
-    }
-    if (!null && nk > 0) {
-      // c_k = tau (d_k + conj(vh) h_k) for the trailing columns k = j+1 ..
-      for (int k = threadIdx.x; k < nk; k += NT) {
-        const int sl = 4 * (k + 1);
-        const double dr = redo[sl] + (vh.x * redo[sl + 2] + vh.y * redo[sl + 3]);
-        const double di = redo[sl + 1] + (vh.x * redo[sl + 3] - vh.y * redo[sl + 2]);
-        qs.coef[k] = make_double2(tau * dr, tau * di);
-      }
-      __syncthreads();
-      pc.lap(P.ctl, 13);
-      // update the trailing columns on the own rows r >= j
-      const long long r0 = max(rb, (long long)j);
-      const int nrr = (int)max(0LL, re - r0);
-      const float inv_nrr = nrr > 0 ? 1.0f / (float)nrr : 0.0f;
-      for (int idx = threadIdx.x; idx < nk * nrr; idx += NT) {
-        const int k = fdivu(idx, nrr, inv_nrr);
-        const long long r = r0 + (idx - k * nrr);
-        const double2 vr = (r == j) ? vh : WA(j, r);
-        const double2 ck = qs.coef[k];
-        double2* wp = &WA(j + 1 + k, r);
-        double2 w = *wp;
-        w.x -= vr.x * ck.x - vr.y * ck.y;
-        w.y -= vr.x * ck.y + vr.y * ck.x;
-        *wp = w;
-      }
-    }
-    if (nk > 0) {
-      __syncthreads();  // the updates (pair mapping) before the next column's dots (lane mapping)
-      pc.lap(P.ctl, 14);
-      double* mine = red[rp];
-      rp ^= 1;
-      prepare(j + 1, mine);
-      pc.lap(P.ctl, 15);
-      team_reduce_vec(tm, mine, redo, 4 * nk);
-      pc.lap(P.ctl, 9);
-    }
-  }
-  __syncthreads();
-  if (in_smem) {  // rows < n to the global workspace (read across CTAs below)
-    const long long rt = min(re, (long long)n);
-    const int ntop = (int)max(0LL, rt - rb);
-    for (int idx = threadIdx.x; idx < n * ntop; idx += NT) {
-      const int c = idx / ntop;
-      const long long r = rb + (idx - c * ntop);
-      W[(long long)c * rows + r] = WA(c, r);
-    }
-  }
-  pc.lap(P.ctl, 9);
-  // Compact WY form Q = I - Vh T Vh^H, built from the unit-norm reflectors vh_j = v_j / |v_j|
-  // (tau = 2): a column just above the null threshold has |v_j| ~ 1e-8 |M| and tau_j ~ 1e16,
-  // and the unnormalised form would chain such factors through T and lose orthogonality.
-  // Gram of the unit reflectors: G[a][b] = vh_a^H vh_b over rows r >= max(a, b), a <= b;
-  // per pair a walk over the own rows with two accumulator sets
-  {
-    const int n2 = n * n;
-    double* mine = red[rp];
-    rp ^= 1;
-    for (int pidx = threadIdx.x; pidx < n2; pidx += NT) {
-      const int a = pidx / n, b = pidx - (pidx / n) * n;
-      double g0r = 0, g0i = 0, g1r = 0, g1i = 0;
-      if (a <= b && qs.tau[a] != 0.0 && qs.tau[b] != 0.0) {
-        long long r = max(rb, (long long)b);
-        for (; r + 1 < re; r += 2) {
-          const double2 va0 = (r == a) ? qs.vhead[a] : WA(a, r);
-          const double2 vb0 = (r == b) ? qs.vhead[b] : WA(b, r);
-          const double2 va1 = WA(a, r + 1);
-          const double2 vb1 = (r + 1 == b) ? qs.vhead[b] : WA(b, r + 1);
-          g0r = fma(va0.x, vb0.x, fma(va0.y, vb0.y, g0r));
-          g0i = fma(va0.x, vb0.y, fma(-va0.y, vb0.x, g0i));
-          g1r = fma(va1.x, vb1.x, fma(va1.y, vb1.y, g1r));
-          g1i = fma(va1.x, vb1.y, fma(-va1.y, vb1.x, g1i));
-        }
-        if (r < re) {
-          const double2 va0 = (r == a) ? qs.vhead[a] : WA(a, r);
-          const double2 vb0 = (r == b) ? qs.vhead[b] : WA(b, r);
-          g0r = fma(va0.x, vb0.x, fma(va0.y, vb0.y, g0r));
-          g0i = fma(va0.x, vb0.y, fma(-va0.y, vb0.x, g0i));
-        }
-      }
-      mine[2 * pidx] = g0r + g1r;
-      mine[2 * pidx + 1] = g0i + g1i;
-    }
-    team_reduce_vec(tm, mine, redo, 2 * n2);
-    for (int pidx = threadIdx.x; pidx < n2; pidx += NT) {
-      const int a = pidx / n, b = pidx - (pidx / n) * n;
-      if (a > b) continue;
-      const double sab = qs.shat[a] * qs.shat[b];
-      const double gr = sab * redo[2 * pidx], gi = sab * redo[2 * pidx + 1];
-      G[a * ldg + b] = make_double2(gr, gi);
-      G[b * ldg + a] = make_double2(gr, -gi);
-    }
-    __syncthreads();
-  }
-  pc.lap(P.ctl, 10);
-  // T (upper triangular): T[j][j] = 2, T[0:j, j] = -2 T[0:j, 0:j] G[0:j, j] (rows and columns
-  // of identity reflectors stay zero)
-  for (int idx = threadIdx.x; idx < n * n; idx += NT) Tm[idx / n * ldg + idx % n] = make_double2(0, 0);
-  __syncthreads();
-  for (int j = 0; j < n; ++j) {
-    const double tj = qs.tau[j] != 0.0 ? 2.0 : 0.0;
-    if (threadIdx.x < j && tj != 0.0) {
-      const int i = threadIdx.x;
-      double sr0 = 0, si0 = 0, sr1 = 0, si1 = 0;  // two chains (FP64 latency)
-      int k = i;
-      for (; k + 1 < j; k += 2) {
-        const double2 t0 = Tm[i * ldg + k], g0 = G[k * ldg + j];
-        const double2 t1 = Tm[i * ldg + k + 1], g1 = G[(k + 1) * ldg + j];
-        sr0 = fma(t0.x, g0.x, fma(-t0.y, g0.y, sr0));
-        si0 = fma(t0.x, g0.y, fma(t0.y, g0.x, si0));
-        sr1 = fma(t1.x, g1.x, fma(-t1.y, g1.y, sr1));
-        si1 = fma(t1.x, g1.y, fma(t1.y, g1.x, si1));
-      }
-      if (k < j) {
-        const double2 t0 = Tm[i * ldg + k], g0 = G[k * ldg + j];
-        sr0 = fma(t0.x, g0.x, fma(-t0.y, g0.y, sr0));
-        si0 = fma(t0.x, g0.y, fma(t0.y, g0.x, si0));
-      }
-      Tm[i * ldg + j] = make_double2(-tj * (sr0 + sr1), -tj * (si0 + si1));
-    }
-    if (threadIdx.x == 0) Tm[j * ldg + j] = make_double2(tj, 0.0);
-    __syncthreads();
-  }
-  // Z[j][c] = shat_j sum_{j <= i <= c} T[j][i] shat_i conj(V[c][i]), so that
-  // Q = I - V Z with the unnormalised V stored in the workspace
-  for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-    const int j = idx / n, c = idx % n;
-    double zr = 0, zi = 0;
-    for (int i = j; i <= c; ++i) {
-      if (qs.tau[i] == 0.0) continue;
-      const double2 t = Tm[j * ldg + i];
-      const double2 v = (c == i) ? qs.vhead[i] : W[(long long)i * rows + c];
-      const double si = qs.shat[i];
-      const double2 vci = make_double2(si * v.x, si * v.y);
-      zr += t.x * vci.x + t.y * vci.y;
-      zi += t.y * vci.x - t.x * vci.y;
-    }
-    Z[j * ldg + c] = make_double2(qs.shat[j] * zr, qs.shat[j] * zi);
-  }
-  pc.lap(P.ctl, 11);
-  // phases of the diagonal of R
-  for (int j = threadIdx.x; j < n; j += NT) {
-    const double2 a = qs.rdiag[j];
-    const double aa = sqrt(a.x * a.x + a.y * a.y);
-    qs.ph[j] = aa > 0.0 ? make_double2(a.x / aa, a.y / aa) : make_double2(1.0, 0.0);
-  }
-  __syncthreads();
-  // R (row j scaled by conj(ph_j)) into the bond buffer: R[j][k] = W[k][j] (k > j), diag alpha_j,
-  // rescaled to ||R||_F = ||M||_F (the weight of dropped sub-columns returns to the kept content)
-  if (tm.rank == 0) {
-    __shared__ double s_rn[NWARP];
-    double loc = 0.0;
-    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-      const int j = idx / n, k = idx % n;
-      double2 r = make_double2(0, 0);
-      if (k > j) r = W[(long long)k * rows + j];
-      else if (k == j) r = qs.rdiag[j];
-      loc = fma(r.x, r.x, fma(r.y, r.y, loc));
-    }
-    loc = warp_sum(loc);
-    if (lane == 0) s_rn[warp] = loc;
-    __syncthreads();
-    double rn = 0.0;
-    for (int w = 0; w < NWARP; ++w) rn += s_rn[w];
-    const double scale = rn > 0.0 ? fro_m / sqrt(rn) : 1.0;
-    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-      const int j = idx / n, k = idx % n;
-      double2 r = make_double2(0, 0);
-      if (k > j) r = W[(long long)k * rows + j];
-      else if (k == j) r = qs.rdiag[j];
-      const double2 p = qs.ph[j];
-      Rout[idx] = make_double2(scale * (r.x * p.x + r.y * p.y), scale * (r.y * p.x - r.x * p.y));
-    }
-  }
-  // Q[r][c] = (delta_rc - sum_j V[r][j] Z[j][c]) * ph_c over the own rows, one (c, r) pair
-  // per thread, written back into the tensor; V[r][j] = 0 for j > r and Z[j][c] = 0 for
-  // j > c, so j runs to min(r, c)
-  for (int idx = threadIdx.x; idx < n * nr; idx += NT) {
-    const int c = fdivu(idx, nr, inv_nr);
-    const long long r = rb + (idx - c * nr);
-    const int jmax = (int)(r < (long long)c ? r : (long long)c);
-    double qre = (r == c) ? 1.0 : 0.0, qim = 0.0;
-    for (int j = 0; j <= jmax; ++j) {
-      if (qs.tau[j] == 0.0) continue;
-      const double2 vr = (r == j) ? qs.vhead[j] : WA(j, r);
-      const double2 z = Z[j * ldg + c];
-      qre -= vr.x * z.x - vr.y * z.y;
-      qim -= vr.x * z.y + vr.y * z.x;
-    }
-    const double2 p = qs.ph[c];
-    A[qr_addr(nd, l, r, c)] = make_double2(qre * p.x - qim * p.y, qre * p.y + qim * p.x);
-  }
-  team_sync(tm);
-  pc.lap(P.ctl, 12);
-}
-
-#include "qr_ds.cuh"
+#include "qr.cuh"
 
 // ------------------------------------------------------------------ absorb
 // A_u <- R applied on leg I.leg (FP64), through a temporary
@@ -1903,6 +1495,43 @@ __device__ __noinline__ void op_absorb(const KernelParams& P, Team& tm, const In
   }
   team_sync(tm);
   for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) A[idx] = work[idx];
+  team_sync(tm);
+}
+
+// A_u <- R applied on leg I.leg (the gauge absorb of the mixed modes) in double-single: the
+// tensor is converted once into the workspace, R into shared memory, every element is a
+// compensated dot of length dims[leg], and the result is written back in FP64.
+__device__ __noinline__ void op_absorb_ds(const KernelParams& P, Team& tm, const Instr& I, double2* work) {
+  const NodeDesc nd = P.nodes[I.node];
+  const long long N = nd.size;
+  double2* A = P.pool + nd.off;
+  const double2* R = P.pool + P.trees[I.tree].bond_off;
+  const int l = I.leg;
+  const int D = nd.dims[l];
+  const int st = nd.strides[l];
+  float4* Ad = reinterpret_cast<float4*>(work);
+  float4* Rd = reinterpret_cast<float4*>(dyn_smem);  // D x D <= 64 KB
+  for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) Ad[idx] = ds_cfrom(A[idx]);
+  for (int k = threadIdx.x; k < D * D; k += NT) Rd[k] = ds_cfrom(R[k]);
+  team_sync(tm);
+  for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
+    const LegPos lp = leg_pos(nd, l, idx);
+    const float4* row = Rd + lp.i * D;
+    const float4* xp = Ad + lp.base;
+    DsAcc ar0, ai0, ar1, ai1;
+    ar0.init(make_float2(0.f, 0.f));
+    ai0.init(make_float2(0.f, 0.f));
+    ar1.init(make_float2(0.f, 0.f));
+    ai1.init(make_float2(0.f, 0.f));
+    int k = 0;
+    for (; k + 1 < D; k += 2) {
+      ds_cmac(ar0, ai0, row[k], xp[(long long)k * st]);
+      ds_cmac(ar1, ai1, row[k + 1], xp[(long long)(k + 1) * st]);
+    }
+    if (k < D) ds_cmac(ar0, ai0, row[k], xp[(long long)k * st]);
+    const float2 r = ds_add(ar0.val(), ar1.val()), i = ds_add(ai0.val(), ai1.val());
+    A[idx] = make_double2(ds_to(r), ds_to(i));
+  }
   team_sync(tm);
 }
 
@@ -2089,19 +1718,19 @@ __device__ void exec_op(const KernelParams& P, Team& tm, const Instr& I, double2
         op_expm<T>(P, tm, I, work, tau);
       break;
     case OP_QR:
-      if (P.precision != 0)
-        op_qr_ds(P, tm, I, work);
+      if constexpr (std::is_same<T, double>::value)
+        op_qr<QrF64>(P, tm, I, work);
       else
-        op_qr(P, tm, I, work);
+        op_qr<QrDs>(P, tm, I, work);
       break;
     case OP_ENV:
       op_env<T>(P, tm, I, work);
       break;
     case OP_ABSORB:
-      if (P.precision != 0)
-        op_absorb_ds(P, tm, I, work);
-      else
+      if constexpr (std::is_same<T, double>::value)
         op_absorb(P, tm, I, work);
+      else
+        op_absorb_ds(P, tm, I, work);
       break;
     case OP_RECORD:
       op_record(P, tm, I, P.traj_count + I.tree);
