@@ -5,12 +5,19 @@
 // (Introduction).  These kernels are the training and inference engine of this library's
 // surrogate, with the plain TTNS sweep as its fallback.
 //
-// Layer product C = op(A) op(B) on tcgen05, M tiles of 128 rows and N tiles of 128 columns
-// per CTA, K in chunks of four MMA K steps.  Every K step accumulates into its own TMEM
-// columns and the steps are summed in shared memory in FP32 round-to-nearest (the tensor
+// Layer product C = op(A) op(B) on tcgen05, one tile of 128 rows and NP = 32 or 64 columns per
+// CTA, optionally with K split over the CTAs of a cluster.  Every MMA K step accumulates into
+// its own TMEM columns and the steps are summed in registers in FP32 round-to-nearest (the tensor
 // core's own FP32 accumulation rounds toward zero, about -0.4 ulp per instruction):
 //   kind 1 (TF32X3): FP32-level products for training;
 //   kind 3 (BF16X1): one BF16 product, for inference.
+//
+// What bounds it: latency.  The products here are small (a 256 x 256 x 256 layer is 34 MFLOP), so
+// a CTA's own chain (load, split, MMA, read back, store) is the time, and the split decides how
+// many SMs share it: 128 x 128 tiles ran that layer on 4 CTAs with scalar loads.  The tile is
+// narrowed, then K is split, until the grid covers most of the 152 SMs; operands are loaded 16
+// bytes at a time and written as whole 16-byte core-matrix rows.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -20,15 +27,16 @@
 #include "../../include/ttns.h"
 #include "tc.cuh"
 
+namespace cg = cooperative_groups;
+
 namespace ttns {
 void set_last_error(const std::string& msg);
 
 namespace {
 constexpr int kNT = 256;
-constexpr int kTM = 128;         // rows per CTA (MMA M)
-constexpr int kTN = 128;         // columns per CTA (MMA N)
-constexpr int kTmem = 512;
-constexpr int kSlots = kTmem / kTN;  // K steps per chunk, one accumulator each
+constexpr int kTM = 128;             // rows per CTA (MMA M)
+constexpr int kTmem = 256;           // tensor-memory columns per CTA (two CTAs fit an SM)
+constexpr int kSplitMax = 4;
 
 // status word of the layer products (TTNS_E_TIMEOUT when a completion wait gave up); a
 // file-scope device variable, so that no call allocates (the calls can be captured in a graph)
@@ -47,64 +55,142 @@ struct GemmArgs {
   long long spin_limit;
 };
 
+// Stages rows [r0, r0 + R) x k in [k0, k0 + kn) of an operand as K-major split planes.  Element
+// (r, k) is X[r * ld + k] (kmaj) or X[k * ld + r]; outside rmax x kmax it is zero.  An item is one
+// 16-byte core-matrix row of E = 16 / esize values along k (kmaj), or four rows of them.  vec: 16-
+// byte loads are aligned (base, ld and k0, r0 are multiples of four floats).
 template <int KIND>
-__global__ void __launch_bounds__(kNT, 1) k_mlp_gemm(GemmArgs g) {
+__device__ __forceinline__ void stage_operand(unsigned char* dst, uint32_t plane, const float* X, int ld, bool kmaj,
+                                              bool vec, int r0, int R, int rmax, int k0, int kn, int kmax) {
   using S = tc::Split<KIND>;
+  constexpr int E = 16 / S::esize;
+  const int nkg = kn / E;
+  auto put = [&](int r, int kg, const float* v) {  // E values of row r
+    unsigned char* o = dst + (uint32_t)((r >> 3) * nkg + kg) * 128u + (uint32_t)(r & 7) * 16u;
+    if constexpr (KIND == tc::KIND_TF32X3) {
+      float h[4], l[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        h[q] = tc::to_tf32(v[q]);
+        l[q] = tc::to_tf32(v[q] - h[q]);
+      }
+      *reinterpret_cast<float4*>(o) = make_float4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<float4*>(o + plane) = make_float4(l[0], l[1], l[2], l[3]);
+    } else {
+      __nv_bfloat162 b[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) b[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+      *reinterpret_cast<uint4*>(o) = *reinterpret_cast<uint4*>(b);
+    }
+  };
+  if (kmaj) {
+    // consecutive threads: 8 rows, then k groups (whole 128-byte blocks in shared memory)
+    for (int it = threadIdx.x; it < R * nkg; it += kNT) {
+      const int r8 = it & 7, kg = (it >> 3) % nkg, rb = (it >> 3) / nkg;
+      const int r = rb * 8 + r8, row = r0 + r, k = k0 + kg * E;
+      float v[E];
+      const float* src = X + (long long)row * ld + k;
+      if (vec && row < rmax && k + E <= kmax) {
+#pragma unroll
+        for (int q = 0; q < E; q += 4) {
+          const float4 f = *reinterpret_cast<const float4*>(src + q);
+          v[q] = f.x;
+          v[q + 1] = f.y;
+          v[q + 2] = f.z;
+          v[q + 3] = f.w;
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < E; ++q) v[q] = (row < rmax && k + q < kmax) ? src[q] : 0.0f;
+      }
+      put(r, kg, v);
+    }
+  } else {
+    // consecutive threads: groups of four rows (contiguous in memory), then k groups
+    const int nr4 = R / 4;
+    for (int it = threadIdx.x; it < nr4 * nkg; it += kNT) {
+      const int r = 4 * (it % nr4), kg = it / nr4;
+      const int row = r0 + r, k = k0 + kg * E;
+      float v[4][E];
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        const float* src = X + (long long)(k + q) * ld + row;
+        float f[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (k + q < kmax) {
+          if (vec && row + 4 <= rmax) {
+            const float4 x = *reinterpret_cast<const float4*>(src);
+            f[0] = x.x;
+            f[1] = x.y;
+            f[2] = x.z;
+            f[3] = x.w;
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (row + i < rmax) f[i] = src[i];
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i][q] = f[i];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) put(r + i, kg, v[i]);
+    }
+  }
+}
+
+// K steps per chunk: one accumulator of NP columns each
+template <int NP>
+__host__ __device__ constexpr int chunk_steps() {
+  return kTmem / NP;
+}
+
+template <int KIND, int NP>
+__global__ void __launch_bounds__(kNT, 2) k_mlp_gemm(GemmArgs g) {
+  using S = tc::Split<KIND>;
+  constexpr int KS = S::kstep;
+  constexpr int kSteps = chunk_steps<NP>();
+  constexpr int chunk = kSteps * KS;
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint64_t mbar;
   __shared__ uint32_t tbase_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * kTM, n0 = blockIdx.y * kTN;
-  const int nn = min(kTN, g.N - n0);
-  const int Npad = ((nn + 15) / 16) * 16;  // MMA N for this tile
-  constexpr int KS = S::kstep;
-  const int chunk = kSlots * KS;           // real K per chunk
-  const int ktot = ((g.K + KS - 1) / KS) * KS;
-  const int ldsum = kTN + 1;
-  float* sums = reinterpret_cast<float*>(sm);
-  const uint32_t sum_bytes = ((uint32_t)kTM * ldsum * 4u + 1023u) & ~1023u;
-  const uint32_t a_plane = (uint32_t)kTM * chunk * S::esize;
-  const uint32_t b_plane = (uint32_t)kTN * chunk * S::esize;
-  unsigned char* Ap = sm + sum_bytes;
-  unsigned char* Bp = Ap + S::parts * a_plane;
+  const int split = gridDim.z;  // = cluster size along z
+  const int m0 = blockIdx.x * kTM, n0 = blockIdx.y * NP;
+  // this CTA's part of K: whole K steps
+  const int steps = (g.K + KS - 1) / KS, per = (steps + split - 1) / split;
+  const int kbeg = min(g.K, (int)blockIdx.z * per * KS);
+  const int kend = min(g.K, kbeg + per * KS);
+  constexpr uint32_t a_plane = (uint32_t)kTM * chunk * S::esize;
+  constexpr uint32_t b_plane = (uint32_t)NP * chunk * S::esize;
+  constexpr int ldo = NP + 1;
+  float* out = reinterpret_cast<float*>(sm);  // the tile's partial result, after the last MMA
+  unsigned char* Ap = sm;
+  unsigned char* Bp = sm + S::parts * a_plane;
   if (warp == 0) tc::tmem_alloc(&tbase_s, kTmem);
   if (tid == 0) tc::mbar_init(&mbar, 1);
+  const bool va = g.lda % 4 == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
+  const bool vb = g.ldb % 4 == 0 && (reinterpret_cast<uintptr_t>(g.B) & 15) == 0;
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tbase = tbase_s;
   const int q4 = warp & 3, half = warp >> 2, my_row = q4 * 32 + lane;
-  const int c_lo = half * (Npad / 2), c_hi = c_lo + Npad / 2;
-  for (int c = c_lo; c < c_hi; ++c) sums[my_row * ldsum + c] = 0.0f;
+  float acc[NP / 2];  // row my_row, columns half * NP / 2 ..
+#pragma unroll
+  for (int c = 0; c < NP / 2; ++c) acc[c] = 0.0f;
   uint32_t phase = 0;
   bool ok = true;
-  for (int k0 = 0; k0 < ktot && ok; k0 += chunk) {
-    const int kn = min(chunk, ktot - k0);   // a multiple of KS
-    // A tile: kTM rows x kn; consecutive threads take consecutive rows (transA) or k
-    for (int idx = tid; idx < kTM * kn; idx += kNT) {
-      int r, k;
-      if (g.transA) { r = idx % kTM; k = idx / kTM; } else { k = idx % kn; r = idx / kn; }
-      const int m = m0 + r, kk = k0 + k;
-      float v = 0.0f;
-      if (m < g.M && kk < g.K) v = g.transA ? g.A[(long long)kk * g.lda + m] : g.A[(long long)m * g.lda + kk];
-      tc::put_split_f<KIND>(Ap, a_plane, r, k, kn, v);
-    }
-    // B tile as N x K (K-major): element (n, k) = B(k, n)
-    for (int idx = tid; idx < Npad * kn; idx += kNT) {
-      int c, k;
-      if (g.transB) { k = idx % kn; c = idx / kn; } else { c = idx % Npad; k = idx / Npad; }
-      const int n = n0 + c, kk = k0 + k;
-      float v = 0.0f;
-      if (c < nn && kk < g.K) v = g.transB ? g.B[(long long)n * g.ldb + kk] : g.B[(long long)kk * g.ldb + n];
-      tc::put_split_f<KIND>(Bp, b_plane, c, k, kn, v);
-    }
+  for (int k0 = kbeg; k0 < kend && ok; k0 += chunk) {
+    const int kn = min(chunk, ((kend - k0 + KS - 1) / KS) * KS);
+    stage_operand<KIND>(Ap, a_plane, g.A, g.lda, !g.transA, va, m0, kTM, g.M, k0, kn, kend);
+    stage_operand<KIND>(Bp, b_plane, g.B, g.ldb, g.transB != 0, vb, n0, NP, g.N, k0, kn, kend);
     tc::fence_proxy_async();
     __syncthreads();
     const int nsteps = kn / KS;
     if (tid == 0) {
       tc::fence_after();
       for (int ks = 0; ks < nsteps; ++ks)
-        tc::issue_kstep<KIND>(tbase + (uint32_t)(ks * Npad), Ap, a_plane, Bp, b_plane, Npad, kn, ks);
+        tc::issue_kstep<KIND>(tbase + (uint32_t)(ks * NP), Ap, a_plane, Bp, b_plane, NP, kn, ks);
       tc::commit(&mbar);
     }
     const bool w = tc::mbar_wait(&mbar, phase, g.spin_limit);
@@ -112,42 +198,56 @@ __global__ void __launch_bounds__(kNT, 1) k_mlp_gemm(GemmArgs g) {
     ok = __syncthreads_and(w) != 0;
     if (!ok) break;
     phase ^= 1u;
-    const uint32_t lane_base = tbase + ((uint32_t)(q4 * 32) << 16);
-    for (int c = c_lo; c < c_hi; c += 8) {
-      float acc[8];
+    const uint32_t lane_base = tbase + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(half * (NP / 2));
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
-      for (int ks = 0; ks < nsteps; ++ks) {
-        float v[8];
-        tc::tmem_ld8(lane_base + (uint32_t)(ks * Npad + c), v);
+    for (int c = 0; c < NP / 2; c += 8) {
+      uint32_t r[kSteps][8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] += v[j];
-      }
+      for (int ks = 0; ks < kSteps; ++ks)
+        if (ks < nsteps) tc::tmem_ld8_nowait(lane_base + (uint32_t)(ks * NP + c), r[ks]);
+      tc::tmem_wait_ld();
 #pragma unroll
-      for (int j = 0; j < 8; ++j) sums[my_row * ldsum + c + j] += acc[j];
+      for (int ks = 0; ks < kSteps; ++ks)
+        if (ks < nsteps) {
+          tc::tmem_pin8(r[ks]);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[c + j] += __uint_as_float(r[ks][j]);
+        }
     }
     tc::fence_before();
     __syncthreads();
   }
-  if (ok) {
-    // epilogue: rows of the tile, columns coalesced (one column per thread, rows in turn)
-    for (int idx = tid; idx < kTM * nn; idx += kNT) {
-      const int r = idx / nn, c = idx % nn;
-      const int m = m0 + r, n = n0 + c;
-      if (m >= g.M) continue;
-      float v = sums[r * ldsum + c];
-      if (g.epi == 1 || g.epi == 2) v += g.aux[n];
-      if (g.epi == 2) v = tanhf(v);
-      if (g.epi == 3) {
-        const float h = g.aux[(long long)m * g.ldc + n];
-        v *= 1.0f - h * h;
-      }
-      g.C[(long long)m * g.ldc + n] = v;
-    }
-  } else {
+  if (!ok) {
     if (tid == 0) atomicCAS(&g_mlp_status, 0, (int)TTNS_E_TIMEOUT);
     tc::mbar_wait(&mbar, phase, g.spin_limit);  // the MMAs in flight finish before TMEM is released
+    __syncthreads();
   }
+#pragma unroll
+  for (int c = 0; c < NP / 2; ++c) out[my_row * ldo + half * (NP / 2) + c] = acc[c];
+  // the CTAs of a split add their partial tiles in a fixed order, each a share of the rows
+  cg::cluster_group cl = cg::this_cluster();
+  if (split > 1) cl.sync(); else __syncthreads();
+  const int rps = kTM / split, rlo = blockIdx.z * rps;
+  for (int idx = tid; idx < rps * NP; idx += kNT) {
+    const int r = rlo + idx / NP, c = idx % NP;
+    const int m = m0 + r, n = n0 + c;
+    if (m >= g.M || n >= g.N) continue;
+    float v;
+    if (split == 1) {
+      v = out[r * ldo + c];
+    } else {
+      v = *cl.map_shared_rank(out + r * ldo + c, 0);
+      for (int z = 1; z < split; ++z) v += *cl.map_shared_rank(out + r * ldo + c, z);
+    }
+    if (g.epi == 1 || g.epi == 2) v += g.aux[n];
+    if (g.epi == 2) v = tanhf(v);
+    if (g.epi == 3) {
+      const float h = g.aux[(long long)m * g.ldc + n];
+      v *= 1.0f - h * h;
+    }
+    g.C[(long long)m * g.ldc + n] = v;
+  }
+  if (split > 1) cl.sync();  // the peers' tiles are read before their CTAs leave
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
@@ -155,12 +255,29 @@ __global__ void __launch_bounds__(kNT, 1) k_mlp_gemm(GemmArgs g) {
 }
 
 // out[n] = sum_m X[m * ld + n] (bias gradients), fixed order per column
+// (32 columns per block, rows over 8 lanes each, then a fixed tree: one thread per column walked
+// through all rows in 4 blocks)
 __global__ void k_colsum(const float* X, int M, int N, int ld, float* out) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.0f;
-  for (int m = 0; m < M; ++m) s += X[(long long)m * ld + n];
-  out[n] = s;
+  __shared__ float part[8][33];
+  const int c = threadIdx.x & 31, q = threadIdx.x >> 5;
+  const int n = blockIdx.x * 32 + c;
+  float s0 = 0.0f, s1 = 0.0f;
+  if (n < N) {
+    int m = q;
+    for (; m + 8 < M; m += 16) {
+      s0 += X[(long long)m * ld + n];
+      s1 += X[(long long)(m + 8) * ld + n];
+    }
+    if (m < M) s0 += X[(long long)m * ld + n];
+  }
+  part[q][c] = s0 + s1;
+  __syncthreads();
+  if (q == 0 && n < N) {
+    float t[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) t[i] = part[i][c];
+    out[n] = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+  }
 }
 
 // dy = (y - t) * scale
@@ -181,16 +298,48 @@ __global__ void k_adam(float* p, const float* g, float* m, float* v, long long n
   }
 }
 
+template <int KIND, int NP>
+cudaError_t launch_tile(const GemmArgs& g, int split, cudaStream_t st) {
+  using S = tc::Split<KIND>;
+  constexpr size_t planes = (size_t)S::parts * (kTM + NP) * (chunk_steps<NP>() * S::kstep) * S::esize;
+  constexpr size_t tile = (size_t)kTM * (NP + 1) * sizeof(float);
+  // at most two CTAs per SM, so that a CTA never waits for tensor memory while its cluster's
+  // other CTAs hold some
+  constexpr size_t two_per_sm = 80 * 1024;
+  constexpr size_t need = planes > tile ? planes : tile;
+  constexpr size_t smem = need > two_per_sm ? need : two_per_sm;
+  static_assert(2 * kTmem <= 512, "tensor memory of two CTAs");
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_gemm<KIND, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((g.M + kTM - 1) / kTM, (g.N + NP - 1) / NP, split);
+  cfg.blockDim = dim3(kNT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = split;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_mlp_gemm<KIND, NP>, g);
+}
+
+// The widest tile that still gives the chip most of its 152 SMs (each narrowing stages the rows
+// of A once more), then K split in two or four parts of at least four K steps each until there
+// are CTAs for all of them (a CTA's K chunks run one after another).
 template <int KIND>
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t st) {
-  using S = tc::Split<KIND>;
-  const size_t sum_bytes = ((size_t)kTM * (kTN + 1) * 4 + 1023) & ~(size_t)1023;
-  const size_t smem = sum_bytes + (size_t)S::parts * (kTM + kTN) * (kSlots * S::kstep) * S::esize;
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_gemm<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid((g.M + kTM - 1) / kTM, (g.N + kTN - 1) / kTN);
-  k_mlp_gemm<KIND><<<grid, kNT, smem, st>>>(g);
-  return cudaGetLastError();
+  constexpr int kFill = 96, kFillSplit = 160;
+  const long long rt = (g.M + kTM - 1) / kTM;
+  auto ctas = [&](int np) { return rt * ((g.N + np - 1) / np); };
+  const int np = ctas(64) >= kFill ? 64 : 32;
+  const int steps = (g.K + tc::Split<KIND>::kstep - 1) / tc::Split<KIND>::kstep;
+  int split = 1;
+  while (split < kSplitMax && ctas(np) * split < kFillSplit && steps >= 8 * split) split *= 2;
+  if (np == 64) return launch_tile<KIND, 64>(g, split, st);
+  return launch_tile<KIND, 32>(g, split, st);
 }
 }  // namespace
 }  // namespace ttns
@@ -224,7 +373,7 @@ extern "C" ttns_status ttns_mlp_colsum(const float* X, int M, int N, int ld, flo
     set_last_error("ttns_mlp_colsum: bad arguments");
     return TTNS_E_INVALID;
   }
-  ttns::k_colsum<<<(N + 255) / 256, 256, 0, (cudaStream_t)cuda_stream>>>(X, M, N, ld, out);
+  ttns::k_colsum<<<(N + 31) / 32, 256, 0, (cudaStream_t)cuda_stream>>>(X, M, N, ld, out);
   return cudaGetLastError() == cudaSuccess ? TTNS_OK : TTNS_E_CUDA;
 }
 
