@@ -16,22 +16,25 @@ namespace ttns {
 cudaError_t launch_sweep(const KernelParams& P, int phase, int grid, int cluster, int cooperative,
                          cudaStream_t stream);
 cudaError_t max_grid_for(int cluster, long long smem_bytes, int* grid);
-cudaError_t launch_density(const double2* pool, const NodeDesc& nd, int l, const double2* rho_in, double2* xbuf,
-                           double* partials,
-                           int nblocks, double* out, cudaStream_t st);
+cudaError_t launch_density(const double2* pool, const NodeDesc& nd, int l, double* partials, int nblocks, double* out,
+                           cudaStream_t st);
+cudaError_t launch_down(const double2* pool, const NodeDesc* d_nodes, const DownBatch& b, double* obs, double2* xbuf,
+                        long long kvec, double* partials, cudaStream_t st);
+cudaError_t launch_populations(const double2* pool, const NodeDesc* d_nodes, const TreeDesc* d_trees, int n_trees,
+                               double* out, cudaStream_t st);
 cudaError_t launch_energy(const KernelParams& P, int node, int terms, int n2, double* partials, int nblocks,
                           double* out, cudaStream_t st);
-cudaError_t launch_occ(const double2* dens, int d, double* out, cudaStream_t st);
 cudaError_t launch_wait_selftest(Ctl* ctl, long long spin_limit, int skip, cudaStream_t st);
 cudaError_t launch_apply_x(const KernelParams& P, int node, int terms, int n2, const double2* x, double2* y,
-                           int nblocks, cudaStream_t st);
+                           int nblocks, int count, cudaStream_t st);
 cudaError_t launch_herm_jacobi(const double2* base, const long long* offs, const int* ns, const int* lds, int count,
                                int n_max, double* evals, double2* evecs, cudaStream_t st);
 cudaError_t launch_bath_states(const double2* A, long long R, int n_el, const double2* U, const double* sig, int nb,
                                double2* Phi, cudaStream_t st);
-cudaError_t launch_build_x(const double2* Phi, int k, int l, long long R, int n_el, double2* X, cudaStream_t st);
+cudaError_t launch_build_x(const double2* Phi, int c0, int count, long long R, int n_el, double2* X, long long kvec,
+                           cudaStream_t st);
 cudaError_t launch_project(const double2* y, const double2* Phi, long long R, int n_el, int nb, double* partials,
-                           int nblocks, double* out, cudaStream_t st);
+                           int nblocks, double* out, int count, long long kvec, cudaStream_t st);
 cudaError_t launch_sub(const double* a, const double* b, double* c, int n, cudaStream_t st);
 cudaError_t launch_mirror32(const double2* pool, float2* pool32, long long n, cudaStream_t st);
 cudaError_t launch_pad_copy(const double2* src_pool, const NodeDesc& so, double2* dst_pool, const NodeDesc& dn,
@@ -77,7 +80,7 @@ struct ttns_tree {
   double* obs = nullptr;        // observable scratch (partials + outputs)
   long long obs_size = 0;
   // regions of obs (doubles)
-  long long o_bond = 0, o_site = 0, o_occ = 0, o_rho = 0, o_en = 0;
+  long long o_bond = 0, o_occ = 0, o_rho = 0, o_en = 0;
   KernelParams P{};
   std::vector<void*> allocs;
   double t_fs = 0.0;
@@ -412,8 +415,7 @@ static ttns_status device_init(ttns_tree* t) {
   const long long nn = (long long)C.nodes.size();
   const long long d2 = 2LL * C.max_D * C.max_D;
   t->o_bond = 1024LL * d2;
-  t->o_site = t->o_bond + nn * d2;
-  t->o_occ = t->o_site + nn * d2;
+  t->o_occ = t->o_bond + nn * d2;
   // rho_S is read as complex (16-byte loads) by the eigen kernels: 256-byte aligned
   t->o_rho = (t->o_occ + nn + 64 + 31) & ~31LL;
   t->o_en = t->o_rho + 2 * 64 * 64;
@@ -666,13 +668,12 @@ static int find_root_fwd_terms(ttns_tree* t, int tree_idx, int* n2) {
   return -1;
 }
 
-// root densities: rho_S (phys leg) into obs + off
-static ttns_status density(ttns_tree* t, int node, int leg, const double2* rho_in, double* out) {
+// density of a root leg (the centre) into out
+static ttns_status root_density(ttns_tree* t, int node, int leg, double* out) {
   const NodeDesc& nd = t->C.nodes[node];
-  const int D = nd.dims[leg];
-  // about eight rows per block; rho_in applied once per element into the worker workspace
-  int nblocks = (int)std::min<long long>(1024, std::max<long long>(1, nd.size / D / 8));
-  CUDA_TRY(launch_density(t->pool, nd, leg, rho_in, t->work, t->obs, nblocks, out, t->stream));
+  // about eight rows per block
+  const int nblocks = (int)std::min<long long>(1024, std::max<long long>(1, nd.size / nd.dims[leg] / 8));
+  CUDA_TRY(launch_density(t->pool, nd, leg, t->obs, nblocks, out, t->stream));
   return TTNS_OK;
 }
 
@@ -683,7 +684,7 @@ extern "C" ttns_status ttns_reduced_density_matrix(ttns_tree* t, int tree_idx, d
   if (s != TTNS_OK) return s;
   const TreeDesc& td = t->C.trees[tree_idx];
   double* out = t->obs + t->o_rho;
-  if ((s = density(t, td.node0, td.root_phys_leg, nullptr, out)) != TTNS_OK) return s;
+  if ((s = root_density(t, td.node0, td.root_phys_leg, out)) != TTNS_OK) return s;
   CUDA_TRY(cudaMemcpyAsync(rho_out, out, sizeof(double) * 2 * td.n_el * td.n_el, cudaMemcpyDeviceToHost, t->stream));
   CUDA_TRY(cudaStreamSynchronize(t->stream));
   return TTNS_OK;
@@ -707,40 +708,57 @@ extern "C" ttns_status ttns_occupations(ttns_tree* t, int tree_idx, double* occ_
 }
 
 static ttns_status downward_pass(ttns_tree* t, int tree_idx, bool sites) {
-  ttns_status s;
   const HostTree& h = t->C.host[tree_idx];
   const TreeDesc& td = t->C.trees[tree_idx];
-  const int maxD = t->C.max_D;
-  // per node: incoming parent-bond density at dens + v * 2 maxD^2
-  double* dens = t->obs + t->o_bond;
-  double* occ_dev = t->obs + t->o_occ;
-  // preorder walk
-  std::vector<int> order;
-  std::vector<int> stack{0};
-  while (!stack.empty()) {
-    int v = stack.back();
-    stack.pop_back();
-    order.push_back(v);
-    for (auto it = h.children[v].rbegin(); it != h.children[v].rend(); ++it) stack.push_back(*it);
-  }
-  std::vector<int> site_pos(h.n(), -1);
+  const long long d2 = 2LL * t->C.max_D * t->C.max_D;
+  std::vector<int> site_pos(h.n(), -1), depth(h.n(), 0);
   {
     int k = 0;
     for (auto& c : h.chain_nodes)
       for (int v : c) site_pos[v] = k++;
   }
-  double* site_dens = t->obs + t->o_site;  // 2*maxD^2 per site
-  for (int v : order) {
-    const int gv = td.node0 + v;
-    const double2* rin = h.parent[v] >= 0 ? (const double2*)(dens + (long long)v * 2 * maxD * maxD) : nullptr;
-    for (int c : h.children[v]) {
-      if ((s = density(t, gv, h.leg_of(v, c), rin, dens + (long long)c * 2 * maxD * maxD)) != TTNS_OK) return s;
+  // levels of equal depth: their nodes depend on the level above only (parents precede children
+  // in node order)
+  std::vector<std::vector<int>> levels;
+  for (int v = 0; v < h.n(); ++v) {
+    if (h.parent[v] >= 0) depth[v] = depth[h.parent[v]] + 1;
+    if (depth[v] >= (int)levels.size()) levels.resize(depth[v] + 1);
+    levels[depth[v]].push_back(v);
+  }
+  // X = rho_in A goes to the worker workspace: one Krylov slot per node of a batch
+  const int slots = std::min(t->P.mmax, kDownNodes);
+  for (const auto& lev : levels) {
+    DownBatch b{};
+    auto flush = [&]() -> ttns_status {
+      if (b.n_nodes > 0)
+        CUDA_TRY(launch_down(t->pool, t->d_nodes, b, t->obs, t->work, t->P.kvec, t->obs, t->stream));
+      b = DownBatch{};
+      return TTNS_OK;
+    };
+    for (int v : lev) {
+      const int nc = (int)h.children[v].size();
+      const bool site = sites && h.parent[v] >= 0 && h.phys[v] > 0 && site_pos[v] >= 0;
+      if (nc == 0 && !site) continue;
+      if (b.n_nodes == slots || b.n_dens + nc > kDownDens) {
+        ttns_status s = flush();
+        if (s != TTNS_OK) return s;
+      }
+      DownNode& dn = b.node[b.n_nodes];
+      dn.node = td.node0 + v;
+      dn.rho_in = h.parent[v] >= 0 ? t->o_bond + v * d2 : -1;
+      dn.occ = site ? t->o_occ + site_pos[v] : -1;
+      dn.size = t->C.nodes[dn.node].size;
+      for (int c : h.children[v]) {
+        DownDens& dd = b.dens[b.n_dens++];
+        dd.item = b.n_nodes;
+        dd.leg = h.leg_of(v, c);
+        dd.D = h.bond[c];
+        dd.out = t->o_bond + c * d2;
+      }
+      ++b.n_nodes;
     }
-    if (sites && h.parent[v] >= 0 && h.phys[v] > 0 && site_pos[v] >= 0) {
-      double* sd = site_dens + (long long)site_pos[v] * 2 * maxD * maxD;
-      if ((s = density(t, gv, h.phys_leg(v), rin, sd)) != TTNS_OK) return s;
-      CUDA_TRY(launch_occ((const double2*)sd, h.phys[v], occ_dev + site_pos[v], t->stream));
-    }
+    ttns_status s = flush();
+    if (s != TTNS_OK) return s;
   }
   return TTNS_OK;
 }
@@ -809,17 +827,17 @@ extern "C" ttns_status ttns_energy_surfaces(ttns_tree* t, int tree_idx, double s
   const NodeDesc& rootd = t->C.nodes[td.node0];
   const long long R = rootd.size / ne;
   // scratch: evals (2 x 64), evecs (64 x 64 complex), U and sigma of the kept states, H / T / V
-  // (32 x 32 complex each), projection partials (256 blocks x 2 x 32), offsets and sizes
+  // (32 x 32 complex each), projection partials (16 columns x 32 blocks x 2 x 32), offsets and sizes
   const long long o_ev = 0, o_vec = 128, o_u = o_vec + 2 * 64 * 64, o_sig = o_u + 2 * 16 * 16,
                   o_h = o_sig + 64, o_t = o_h + 2 * 32 * 32, o_v = o_t + 2 * 32 * 32, o_part = o_v + 2 * 32 * 32,
-                  o_offs = o_part + 256 * 2 * 32, o_ns = o_offs + 8, total = o_ns + 8;
+                  o_offs = o_part + 16 * 32 * 2 * 32, o_ns = o_offs + 8, total = o_ns + 8;
   if ((s = surface_scratch(t, total)) != TTNS_OK) return s;
   double* sc = t->surf;
   // 1. environment blocks of the kinetic energy at the current state
   if ((s = kinetic_envs(t)) != TTNS_OK) return s;
   // 2. Schmidt decomposition through rho_S = A^T conj(A): eigenvectors and values
   double* rho = t->obs + t->o_rho;
-  if ((s = density(t, td.node0, td.root_phys_leg, nullptr, rho)) != TTNS_OK) return s;
+  if ((s = root_density(t, td.node0, td.root_phys_leg, rho)) != TTNS_OK) return s;
   if ((s = eig_batch(t, (const double2*)rho, {0}, {ne}, sc + o_ev, (double2*)(sc + o_vec), (long long*)(sc + o_offs),
                      (int*)(sc + o_ns))) != TTNS_OK)
     return s;
@@ -848,20 +866,24 @@ extern "C" ttns_status ttns_energy_surfaces(ttns_tree* t, int tree_idx, double s
   CUDA_TRY(cudaMemcpyAsync(sc + o_u, U.data(), sizeof(double2) * U.size(), cudaMemcpyHostToDevice, t->stream));
   CUDA_TRY(cudaMemcpyAsync(sc + o_sig, sg.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, t->stream));
   // 3. bath states and the projected H_eff(root), T_eff(root) in the basis |phi_k, l>
+  //    (columns in batches: inputs and results in the Krylov slots; an operator with two-stage
+  //    terms has temporaries for one vector only)
   const long long kv = t->P.kvec;
-  double2* slot = t->work + (long long)(t->P.mmax + t->P.n_tmp + 2) * kv;
-  double2 *Phi = slot, *X = slot + kv, *Y = slot + 2 * kv;
+  double2* Phi = t->work + (long long)(t->P.mmax + t->P.n_tmp + 2) * kv;
   const double2* A = t->pool + rootd.off;
   CUDA_TRY(launch_bath_states(A, R, ne, (const double2*)(sc + o_u), sc + o_sig, nb, Phi, t->stream));
-  const int nbl = (int)std::min<long long>(1024, (rootd.size + 255) / 256);
-  const int npb = (int)std::min<long long>(256, R / 64 + 1);
+  const int npb = (int)std::min<long long>(32, R / 64 + 1);
   const int n2h = t->C.lists[td.heff_terms].n2, n2t = t->C.lists[td.teff_terms].n2;
-  for (int c = 0; c < nv; ++c) {
-    CUDA_TRY(launch_build_x(Phi, c / ne, c % ne, R, ne, X, t->stream));
-    CUDA_TRY(launch_apply_x(t->P, td.node0, td.heff_terms, n2h, X, Y, nbl, t->stream));
-    CUDA_TRY(launch_project(Y, Phi, R, ne, nb, sc + o_part, npb, sc + o_h + 2LL * c * nv, t->stream));
-    CUDA_TRY(launch_apply_x(t->P, td.node0, td.teff_terms, n2t, X, Y, nbl, t->stream));
-    CUDA_TRY(launch_project(Y, Phi, R, ne, nb, sc + o_part, npb, sc + o_t + 2LL * c * nv, t->stream));
+  const int batch = n2h > 0 || n2t > 0 ? 1 : std::max(1, std::min({16, t->P.mmax / 2, nv}));
+  const int nbl = (int)std::min<long long>(1024, (rootd.size + 255) / 256);
+  double2 *X = t->work, *Y = t->work + (long long)batch * kv;
+  for (int c = 0; c < nv; c += batch) {
+    const int cnt = std::min(batch, nv - c);
+    CUDA_TRY(launch_build_x(Phi, c, cnt, R, ne, X, kv, t->stream));
+    CUDA_TRY(launch_apply_x(t->P, td.node0, td.heff_terms, n2h, X, Y, nbl, cnt, t->stream));
+    CUDA_TRY(launch_project(Y, Phi, R, ne, nb, sc + o_part, npb, sc + o_h + 2LL * c * nv, cnt, kv, t->stream));
+    CUDA_TRY(launch_apply_x(t->P, td.node0, td.teff_terms, n2t, X, Y, nbl, cnt, t->stream));
+    CUDA_TRY(launch_project(Y, Phi, R, ne, nb, sc + o_part, npb, sc + o_t + 2LL * c * nv, cnt, kv, t->stream));
   }
   // 4. V = H - T and the eigenvalues of both (the matrices are stored by columns: their
   //    transposes, conj(H) and conj(V), have the same eigenvalues)
@@ -891,7 +913,7 @@ static ttns_status bond_spectra(ttns_tree* t, int tree_idx, std::vector<double>*
   const int maxD = t->C.max_D;
   if ((s = downward_pass(t, tree_idx, false)) != TTNS_OK) return s;
   double* rho = t->obs + t->o_rho;
-  if ((s = density(t, td.node0, td.root_phys_leg, nullptr, rho)) != TTNS_OK) return s;
+  if ((s = root_density(t, td.node0, td.root_phys_leg, rho)) != TTNS_OK) return s;
   // matrices: rho_S (root), then every node's parent-bond density
   const long long o_ev = 0, o_offs = 64LL * n, o_ns = o_offs + n + 8, total = o_ns + n + 8;
   if ((s = surface_scratch(t, std::max<long long>(total, 1))) != TTNS_OK) return s;
@@ -1113,18 +1135,7 @@ extern "C" ttns_status ttns_trajectory(ttns_tree* t, int tree_idx, double* out, 
 
 extern "C" ttns_status ttns_populations_device(ttns_tree* t, double* dev_out) {
   if (!t || !dev_out) return fail(TTNS_E_INVALID, "NULL argument");
-  ttns_status s;
-  int off = 0;
-  for (size_t k = 0; k < t->C.trees.size(); ++k) {
-    const TreeDesc& td = t->C.trees[k];
-    double* tmp = t->obs + t->o_rho;
-    if ((s = density(t, td.node0, td.root_phys_leg, nullptr, tmp)) != TTNS_OK) return s;
-    // diagonal (real parts) -> dev_out
-    for (int q = 0; q < td.n_el; ++q)
-      CUDA_TRY(cudaMemcpyAsync(dev_out + off + q, tmp + 2 * (q * td.n_el + q), sizeof(double), cudaMemcpyDeviceToDevice,
-                               t->stream));
-    off += td.n_el;
-  }
+  CUDA_TRY(launch_populations(t->pool, t->d_nodes, t->d_trees, (int)t->C.trees.size(), dev_out, t->stream));
   return TTNS_OK;
 }
 

@@ -171,4 +171,24 @@ struct KernelParams {
   double qr_cutoff;        // relative null threshold of the QR
 };
 
+// One level (or a part of one) of the downward pass of bond densities: the nodes, and the
+// child-bond densities taken from them.  Offsets are in doubles of the observables buffer.
+constexpr int kDownNodes = 16, kDownDens = 32;
+struct DownNode {
+  int node;           // global node index
+  int size;
+  long long rho_in;   // incoming parent-bond density (-1: the root)
+  long long occ;      // <n> of the node's physical leg (-1: not wanted)
+};
+struct DownDens {
+  int item;           // index into DownBatch::node
+  int leg, D;
+  long long out;
+};
+struct DownBatch {
+  int n_nodes, n_dens;
+  DownNode node[kDownNodes];
+  DownDens dens[kDownDens];
+};
+
 }  // namespace ttns

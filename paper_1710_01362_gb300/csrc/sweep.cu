@@ -21,6 +21,7 @@
 
 #include "internal.h"
 #include "ds.cuh"
+#include "index.cuh"
 #include "tc.cuh"
 
 namespace cg = cooperative_groups;
@@ -306,18 +307,6 @@ __device__ void team_finish_multi(Team& tm, int nval, double* out, double scale)
 
 // ------------------------------------------------------------------ sum-of-products apply
 // Position decomposition of flat index idx along leg l.
-// n / d for 0 <= n < 2^24 through a float reciprocal, corrected to the exact quotient
-// (the float estimate is within 2 of it); 64-bit integer division is emulated and slow.
-__device__ __forceinline__ int fdivu(int n, int d, float inv) {
-  int q = __float2int_rz((float)n * inv);
-  int r = n - q * d;
-  if (r < 0) { --q; r += d; }
-  if (r < 0) { --q; r += d; }
-  if (r >= d) { ++q; r -= d; }
-  if (r >= d) { ++q; }
-  return q;
-}
-
 struct LegPos {
   long long base;  // idx - i * stride
   int i;
@@ -1850,35 +1839,9 @@ __global__ void __launch_bounds__(NT, 1) k_sweep(KernelParams P, int phase) {
 }
 
 // ------------------------------------------------------------------ observables
-// Bond or site density of node v's leg l from the incoming parent-bond density rho_in
-// (D_p x D_p, or nullptr at the root):
-//   out[b][b'] = sum rho_in[p', p] A[p, .., b, ..] conj(A[p', .., b', ..]) over the other legs.
-// One CTA per call (small sizes), except that the root (rho_in == nullptr) may be large:
-// a grid of CTAs writes partials, reduced by k_reduce_partials.
-// X = rho_in applied on leg 0 of the node tensor: X[idx] = sum_a' rho_in[a'][a] A[.., a', ..]
-// with a the leg-0 index of idx (the incoming parent-bond density of a downward pass)
-__global__ void k_apply_rho0(const double2* A, NodeDesc nd, const double2* rho_in, double2* X) {
-  const int Dp = nd.dims[0];
-  const long long stp = nd.strides[0];
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < nd.size;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int qa = fdivu((int)idx, (int)stp, nd.inv_strides[0]);
-    const int a = qa - fdivu(qa, Dp, nd.inv_dims[0]) * Dp;
-    const long long b0 = idx - (long long)a * stp;
-    double xr = 0.0, xi = 0.0;
-    for (int a2 = 0; a2 < Dp; ++a2) {
-      const double2 r_ = rho_in[a2 * Dp + a];
-      const double2 v = A[b0 + (long long)a2 * stp];
-      xr = fma(r_.x, v.x, fma(-r_.y, v.y, xr));
-      xi = fma(r_.x, v.y, fma(r_.y, v.x, xi));
-    }
-    X[idx] = make_double2(xr, xi);
-  }
-}
-
-// partials of rho[b][b2] = sum_rows X[row, b] conj(A[row, b2]) along leg l, rows split over
-// the blocks (X = A for the root)
-__global__ void k_density_partial(const double2* X, const double2* A, NodeDesc nd, int l, double* partials) {
+// Density of a root leg: partials of rho[b][b2] = sum_rows A[row, b] conj(A[row, b2]) along leg l,
+// rows split over the blocks
+__global__ void k_density_partial(const double2* A, NodeDesc nd, int l, double* partials) {
   const int D = nd.dims[l];
   const long long N = nd.size;
   const long long st = nd.strides[l];
@@ -1892,7 +1855,7 @@ __global__ void k_density_partial(const double2* X, const double2* A, NodeDesc n
       const long long p = fdivu((int)r, (int)st, nd.inv_strides[l]), q = r - p * st;
       const long long base = p * D * st + q;
       const double2 y = A[base + (long long)b2 * st];
-      const double2 xa = X[base + (long long)b * st];
+      const double2 xa = A[base + (long long)b * st];
       accr = fma(xa.x, y.x, fma(xa.y, y.y, accr));
       acci = fma(xa.y, y.x, fma(-xa.x, y.y, acci));
     }
@@ -1901,20 +1864,14 @@ __global__ void k_density_partial(const double2* X, const double2* A, NodeDesc n
   }
 }
 
+// out[k] = sum of the blocks' partials in a fixed order, one warp per value
 __global__ void k_reduce_partials(const double* partials, int nblocks, int nval, double* out) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nval; k += gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int k = blockIdx.x * nw + (threadIdx.x >> 5); k < nval; k += gridDim.x * nw) {
     double s = 0;
-    for (int b = 0; b < nblocks; ++b) s += partials[(long long)b * nval + k];
-    out[k] = s;
-  }
-}
-
-// <n> = sum_s s Re(rho[s][s]) of one site density
-__global__ void k_occ(const double2* dens, int d, double* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double o = 0;
-    for (int q = 1; q < d; ++q) o += q * dens[q * d + q].x;
-    *out = o;
+    for (int b = lane; b < nblocks; b += 32) s += partials[(long long)b * nval + k];
+    s = warp_sum(s);
+    if (lane == 0) out[k] = s;
   }
 }
 
@@ -1989,10 +1946,13 @@ __global__ void k_stage1_x(KernelParams P, int node, int terms, const double2* x
   }
 }
 
+// (blockIdx.y: vector of a batch, P.kvec apart; more than one only without two-stage terms)
 __global__ void k_apply_x(KernelParams P, int node, int terms, const double2* x, double2* y) {
   const NodeDesc nd = P.nodes[node];
   const TermList L = P.lists[terms];
   OpStage& os = s_os;
+  x += (long long)blockIdx.y * P.kvec;
+  y += (long long)blockIdx.y * P.kvec;
   const int nt = L.count < TTNS_MAX_TERMS ? L.count : TTNS_MAX_TERMS;
   for (int t = threadIdx.x; t < nt; t += blockDim.x) os.terms[t] = P.terms[L.first + t];
   if (threadIdx.x == 0) {
@@ -2007,9 +1967,9 @@ __global__ void k_apply_x(KernelParams P, int node, int terms, const double2* x,
 }
 
 cudaError_t launch_apply_x(const KernelParams& P, int node, int terms, int n2, const double2* x, double2* y,
-                           int nblocks, cudaStream_t st) {
+                           int nblocks, int count, cudaStream_t st) {
   if (n2 > 0) k_stage1_x<<<nblocks, NT, 0, st>>>(P, node, terms, x);
-  k_apply_x<<<nblocks, NT, 0, st>>>(P, node, terms, x, y);
+  k_apply_x<<<dim3(nblocks, count), NT, 0, st>>>(P, node, terms, x, y);
   return cudaGetLastError();
 }
 
@@ -2128,24 +2088,11 @@ cudaError_t max_grid_for(int cluster, long long smem_bytes, int* grid) {
   return cudaSuccess;
 }
 
-cudaError_t launch_density(const double2* pool, const NodeDesc& nd, int l, const double2* rho_in, double2* xbuf,
-                           double* partials, int nblocks, double* out, cudaStream_t st) {
-  const double2* A = pool + nd.off;
-  const double2* X = A;
-  if (rho_in) {
-    long long nb = (nd.size + NT - 1) / NT;
-    nb = nb > 4096 ? 4096 : nb;
-    k_apply_rho0<<<(int)nb, NT, 0, st>>>(A, nd, rho_in, xbuf);
-    X = xbuf;
-  }
-  k_density_partial<<<nblocks, NT, 0, st>>>(X, A, nd, l, partials);
+cudaError_t launch_density(const double2* pool, const NodeDesc& nd, int l, double* partials, int nblocks, double* out,
+                           cudaStream_t st) {
+  k_density_partial<<<nblocks, NT, 0, st>>>(pool + nd.off, nd, l, partials);
   const int D = nd.dims[l];
-  k_reduce_partials<<<(2 * D * D + NT - 1) / NT, NT, 0, st>>>(partials, nblocks, 2 * D * D, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_occ(const double2* dens, int d, double* out, cudaStream_t st) {
-  k_occ<<<1, 32, 0, st>>>(dens, d, out);
+  k_reduce_partials<<<(2 * D * D + NWARP - 1) / NWARP, NT, 0, st>>>(partials, nblocks, 2 * D * D, out);
   return cudaGetLastError();
 }
 
