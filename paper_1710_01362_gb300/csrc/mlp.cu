@@ -36,7 +36,8 @@ namespace {
 constexpr int kNT = 256;
 constexpr int kTM = 128;             // rows per CTA (MMA M)
 constexpr int kTmem = 256;           // tensor-memory columns per CTA (two CTAs fit an SM)
-constexpr int kSplitMax = 4;
+constexpr int kSplitMax = 8;
+constexpr int kGroup = 4;            // K steps added to one partial sum before it joins the total
 
 // status word of the layer products (TTNS_E_TIMEOUT when a completion wait gave up); a
 // file-scope device variable, so that no call allocates (the calls can be captured in a graph)
@@ -53,6 +54,7 @@ struct GemmArgs {
   int epi;          // 0 C = AB, 1 C = AB + bias, 2 C = tanh(AB + bias), 3 C = AB * (1 - aux^2)
   const float* aux; // bias (epi 1, 2: N values) or the layer output h (epi 3: M x N, ldc)
   long long spin_limit;
+  int slots;        // partial sums that a CTA with blockIdx.z > 0 keeps apart
 };
 
 // Stages rows [r0, r0 + R) x k in [k0, k0 + kn) of an operand as K-major split planes.  Element
@@ -156,14 +158,19 @@ __global__ void __launch_bounds__(kNT, 2) k_mlp_gemm(GemmArgs g) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int split = gridDim.z;  // = cluster size along z
   const int m0 = blockIdx.x * kTM, n0 = blockIdx.y * NP;
-  // this CTA's part of K: whole K steps
-  const int steps = (g.K + KS - 1) / KS, per = (steps + split - 1) / split;
+  // this CTA's part of K: whole groups of K steps
+  const int steps = (g.K + KS - 1) / KS;
+  const int per = ((steps + split - 1) / split + kGroup - 1) / kGroup * kGroup;
   const int kbeg = min(g.K, (int)blockIdx.z * per * KS);
   const int kend = min(g.K, kbeg + per * KS);
   constexpr uint32_t a_plane = (uint32_t)kTM * chunk * S::esize;
   constexpr uint32_t b_plane = (uint32_t)NP * chunk * S::esize;
   constexpr int ldo = NP + 1;
-  float* out = reinterpret_cast<float*>(sm);  // the tile's partial result, after the last MMA
+  // The sum runs over groups of four K steps, one group after another from k = 0 whatever the
+  // split is: the CTA of the first part carries a running total, the others keep their groups'
+  // sums apart (in `slots`; with more groups than slots, neighbours share one).
+  float* out = reinterpret_cast<float*>(sm + S::parts * (a_plane + b_plane));
+  const int groups = per / kGroup, gps = (groups + g.slots - 1) / g.slots;
   unsigned char* Ap = sm;
   unsigned char* Bp = sm + S::parts * a_plane;
   if (warp == 0) tc::tmem_alloc(&tbase_s, kTmem);
@@ -178,6 +185,7 @@ __global__ void __launch_bounds__(kNT, 2) k_mlp_gemm(GemmArgs g) {
   float acc[NP / 2];  // row my_row, columns half * NP / 2 ..
 #pragma unroll
   for (int c = 0; c < NP / 2; ++c) acc[c] = 0.0f;
+  int grp = 0;        // groups done
   uint32_t phase = 0;
   bool ok = true;
   for (int k0 = kbeg; k0 < kend && ok; k0 += chunk) {
@@ -200,19 +208,37 @@ __global__ void __launch_bounds__(kNT, 2) k_mlp_gemm(GemmArgs g) {
     phase ^= 1u;
     const uint32_t lane_base = tbase + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(half * (NP / 2));
 #pragma unroll
-    for (int c = 0; c < NP / 2; c += 8) {
-      uint32_t r[kSteps][8];
+    for (int g4 = 0; g4 < kSteps; g4 += kGroup) {
+      if (g4 >= nsteps) break;
 #pragma unroll
-      for (int ks = 0; ks < kSteps; ++ks)
-        if (ks < nsteps) tc::tmem_ld8_nowait(lane_base + (uint32_t)(ks * NP + c), r[ks]);
-      tc::tmem_wait_ld();
+      for (int c = 0; c < NP / 2; c += 8) {
+        uint32_t r[kGroup][8];
 #pragma unroll
-      for (int ks = 0; ks < kSteps; ++ks)
-        if (ks < nsteps) {
-          tc::tmem_pin8(r[ks]);
+        for (int ks = 0; ks < kGroup; ++ks)
+          if (g4 + ks < nsteps) tc::tmem_ld8_nowait(lane_base + (uint32_t)((g4 + ks) * NP + c), r[ks]);
+        tc::tmem_wait_ld();
+        float t[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) acc[c + j] += __uint_as_float(r[ks][j]);
+        for (int j = 0; j < 8; ++j) t[j] = 0.0f;
+#pragma unroll
+        for (int ks = 0; ks < kGroup; ++ks)
+          if (g4 + ks < nsteps) {
+            tc::tmem_pin8(r[ks]);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) t[j] += __uint_as_float(r[ks][j]);
+          }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[c + j] += t[j];
+      }
+      ++grp;
+      if (blockIdx.z > 0 && grp % gps == 0) {
+        float* o = out + (long long)(grp / gps - 1) * (kTM * ldo) + my_row * ldo + half * (NP / 2);
+#pragma unroll
+        for (int c = 0; c < NP / 2; ++c) {
+          o[c] = acc[c];
+          acc[c] = 0.0f;
         }
+      }
     }
     tc::fence_before();
     __syncthreads();
@@ -222,10 +248,21 @@ __global__ void __launch_bounds__(kNT, 2) k_mlp_gemm(GemmArgs g) {
     tc::mbar_wait(&mbar, phase, g.spin_limit);  // the MMAs in flight finish before TMEM is released
     __syncthreads();
   }
+  {  // the total (first part), or the slots not written yet (zero beyond the last group)
+    int sl = blockIdx.z > 0 ? grp / gps : 0;
+    const int nsl = blockIdx.z > 0 ? (groups + gps - 1) / gps : 1;
+    for (; sl < nsl; ++sl) {
+      float* o = out + (long long)sl * (kTM * ldo) + my_row * ldo + half * (NP / 2);
 #pragma unroll
-  for (int c = 0; c < NP / 2; ++c) out[my_row * ldo + half * (NP / 2) + c] = acc[c];
-  // the CTAs of a split add their partial tiles in a fixed order, each a share of the rows
+      for (int c = 0; c < NP / 2; ++c) {
+        o[c] = acc[c];
+        acc[c] = 0.0f;
+      }
+    }
+  }
+  // the CTAs of a split add the parts in order, each a share of the rows
   cg::cluster_group cl = cg::this_cluster();
+  const int nsl = (groups + gps - 1) / gps;
   if (split > 1) cl.sync(); else __syncthreads();
   const int rps = kTM / split, rlo = blockIdx.z * rps;
   for (int idx = tid; idx < rps * NP; idx += kNT) {
@@ -237,7 +274,10 @@ __global__ void __launch_bounds__(kNT, 2) k_mlp_gemm(GemmArgs g) {
       v = out[r * ldo + c];
     } else {
       v = *cl.map_shared_rank(out + r * ldo + c, 0);
-      for (int z = 1; z < split; ++z) v += *cl.map_shared_rank(out + r * ldo + c, z);
+      for (int z = 1; z < split; ++z) {
+        const float* o = cl.map_shared_rank(out + r * ldo + c, z);
+        for (int q = 0; q < nsl; ++q) v += o[q * (kTM * ldo)];
+      }
     }
     if (g.epi == 1 || g.epi == 2) v += g.aux[n];
     if (g.epi == 2) v = tanhf(v);
@@ -255,29 +295,22 @@ __global__ void __launch_bounds__(kNT, 2) k_mlp_gemm(GemmArgs g) {
 }
 
 // out[n] = sum_m X[m * ld + n] (bias gradients), fixed order per column
-// (32 columns per block, rows over 8 lanes each, then a fixed tree: one thread per column walked
-// through all rows in 4 blocks)
-__global__ void k_colsum(const float* X, int M, int N, int ld, float* out) {
-  __shared__ float part[8][33];
-  const int c = threadIdx.x & 31, q = threadIdx.x >> 5;
-  const int n = blockIdx.x * 32 + c;
-  float s0 = 0.0f, s1 = 0.0f;
-  if (n < N) {
-    int m = q;
-    for (; m + 8 < M; m += 16) {
-      s0 += X[(long long)m * ld + n];
-      s1 += X[(long long)(m + 8) * ld + n];
-    }
-    if (m < M) s0 += X[(long long)m * ld + n];
-  }
-  part[q][c] = s0 + s1;
-  __syncthreads();
-  if (q == 0 && n < N) {
-    float t[8];
+// (one thread per column, 16 loads in flight: without them each of the M additions waited for its
+// own load; 32 columns per block, to use more SMs)
+__global__ void __launch_bounds__(32) k_colsum(const float* X, int M, int N, int ld, float* out) {
+  const int n = blockIdx.x * 32 + threadIdx.x;
+  if (n >= N) return;
+  float s = 0.0f;
+  int m = 0;
+  for (; m + 16 <= M; m += 16) {
+    float v[16];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) t[i] = part[i][c];
-    out[n] = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+    for (int i = 0; i < 16; ++i) v[i] = X[(long long)(m + i) * ld + n];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) s += v[i];
   }
+  for (; m < M; ++m) s += X[(long long)m * ld + n];
+  out[n] = s;
 }
 
 // dy = (y - t) * scale
@@ -299,17 +332,19 @@ __global__ void k_adam(float* p, const float* g, float* m, float* v, long long n
 }
 
 template <int KIND, int NP>
-cudaError_t launch_tile(const GemmArgs& g, int split, cudaStream_t st) {
+cudaError_t launch_tile(GemmArgs g, int split, cudaStream_t st) {
   using S = tc::Split<KIND>;
   constexpr size_t planes = (size_t)S::parts * (kTM + NP) * (chunk_steps<NP>() * S::kstep) * S::esize;
   constexpr size_t tile = (size_t)kTM * (NP + 1) * sizeof(float);
   // at most two CTAs per SM, so that a CTA never waits for tensor memory while its cluster's
   // other CTAs hold some
-  constexpr size_t two_per_sm = 80 * 1024;
-  constexpr size_t need = planes > tile ? planes : tile;
-  constexpr size_t smem = need > two_per_sm ? need : two_per_sm;
+  constexpr size_t two_per_sm = 80 * 1024, most = 220 * 1024;
   static_assert(2 * kTmem <= 512, "tensor memory of two CTAs");
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_gemm<KIND, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int steps = (g.K + S::kstep - 1) / S::kstep;
+  const int groups = ((steps + split - 1) / split + kGroup - 1) / kGroup;
+  g.slots = split > 1 ? std::min(groups, (int)((most - planes) / tile)) : 1;
+  const size_t smem = std::max(planes + g.slots * tile, two_per_sm);
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_gemm<KIND, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((g.M + kTM - 1) / kTM, (g.N + NP - 1) / NP, split);
@@ -327,7 +362,7 @@ cudaError_t launch_tile(const GemmArgs& g, int split, cudaStream_t st) {
 }
 
 // The widest tile that still gives the chip most of its 152 SMs (each narrowing stages the rows
-// of A once more), then K split in two or four parts of at least four K steps each until there
+// of A once more), then K split in up to eight parts of at least four K steps each until there
 // are CTAs for all of them (a CTA's K chunks run one after another).
 template <int KIND>
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t st) {
@@ -337,7 +372,7 @@ cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t st) {
   const int np = ctas(64) >= kFill ? 64 : 32;
   const int steps = (g.K + tc::Split<KIND>::kstep - 1) / tc::Split<KIND>::kstep;
   int split = 1;
-  while (split < kSplitMax && ctas(np) * split < kFillSplit && steps >= 8 * split) split *= 2;
+  while (split < kSplitMax && ctas(np) * split < kFillSplit && steps >= 2 * kGroup * split) split *= 2;
   if (np == 64) return launch_tile<KIND, 64>(g, split, st);
   return launch_tile<KIND, 32>(g, split, st);
 }
@@ -358,7 +393,7 @@ extern "C" ttns_status ttns_mlp_gemm(int kind, int M, int N, int K, const float*
     set_last_error("ttns_mlp_gemm: bad kind, size, leading dimension or epilogue");
     return TTNS_E_INVALID;
   }
-  ttns::GemmArgs g{M, N, K, A, lda, transA, B, ldb, transB, C, ldc, epilogue, aux, 20000000000LL};
+  ttns::GemmArgs g{M, N, K, A, lda, transA, B, ldb, transB, C, ldc, epilogue, aux, 20000000000LL, 1};
   cudaStream_t s = (cudaStream_t)cuda_stream;
   cudaError_t e = kind == 1 ? ttns::launch_gemm<ttns::tc::KIND_TF32X3>(g, s) : ttns::launch_gemm<ttns::tc::KIND_BF16X1>(g, s);
   if (e != cudaSuccess) {
@@ -373,7 +408,7 @@ extern "C" ttns_status ttns_mlp_colsum(const float* X, int M, int N, int ld, flo
     set_last_error("ttns_mlp_colsum: bad arguments");
     return TTNS_E_INVALID;
   }
-  ttns::k_colsum<<<(N + 31) / 32, 256, 0, (cudaStream_t)cuda_stream>>>(X, M, N, ld, out);
+  ttns::k_colsum<<<(N + 31) / 32, 32, 0, (cudaStream_t)cuda_stream>>>(X, M, N, ld, out);
   return cudaGetLastError() == cudaSuccess ? TTNS_OK : TTNS_E_CUDA;
 }
 
