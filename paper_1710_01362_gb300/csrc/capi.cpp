@@ -4,8 +4,10 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstddef>
 #include <cstring>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/ttns.h"
@@ -70,6 +72,8 @@ struct ttns_tree {
   Factor* d_chans = nullptr;
   Instr* d_prog = nullptr;
   TreeDesc* d_trees = nullptr;
+  SitePlan* d_sites = nullptr;
+  std::vector<SitePlan> sites;
   Ctl* ctl = nullptr;
   double2* work = nullptr;
   double* red = nullptr;
@@ -359,6 +363,188 @@ static ttns_status wait_and_check(ttns_tree* t, bool phase0, const char* what) {
   return TTNS_OK;
 }
 
+// Plan of an instruction on a site tensor: two or three legs, every dense factor on legs A or C,
+// every row-sparse factor on the remaining leg P (environment updates: A is the instruction's leg
+// and carries no dense factor).  Returns false where the form or the shared memory does not fit;
+// the operation then takes the general path.
+static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize, long long smem, SitePlan* out) {
+  const NodeDesc& nd = C.nodes[I.node];
+  const bool env = I.op == OP_ENV;
+  if ((I.op != OP_FWD && !env) || nd.nl < 2 || nd.nl > 3) return false;
+  const TermList& L = C.lists[I.terms];
+  if (L.n2 > 0 || (env && I.nchan > 16)) return false;
+  struct Pair {
+    int blk;
+    const Factor *d, *s;
+  };
+  std::vector<Pair> prs;
+  auto add = [&](int blk, const Factor* a, const Factor* b) {
+    Pair pr{blk, nullptr, nullptr};
+    for (const Factor* f : {a, b}) {
+      if (!f) continue;
+      const Factor*& slot = f->nnz > 0 ? pr.s : pr.d;
+      if (slot) return false;
+      slot = f;
+    }
+    prs.push_back(pr);
+    return true;
+  };
+  for (int k = 0; k < L.count; ++k) {
+    const Term& T = C.terms[L.first + k];
+    if (!add(0, &T.f[0], T.nf == 2 ? &T.f[1] : nullptr)) return false;
+  }
+  if (env)
+    for (int b = 0; b < I.nchan; ++b)
+      if (!add(1 + b, &C.chans[I.chan_first + b], nullptr)) return false;
+  unsigned dense = 0, sparse = 0;
+  int nj = 0;
+  for (const Pair& pr : prs) {
+    if (pr.d) dense |= 1u << pr.d->leg;
+    if (pr.s) sparse |= 1u << pr.s->leg;
+    nj += pr.s ? pr.s->nnz : 1;
+  }
+  if (nj > kSiteJobs || (sparse & (sparse - 1))) return false;
+  SitePlan sp;
+  std::memset(&sp, 0, sizeof(sp));
+  sp.P = nd.nl - 1;
+  for (int q = 0; q < nd.nl; ++q)
+    if ((sparse >> q) & 1u) sp.P = q;
+  const int l = env ? I.leg : -1;
+  if (((dense >> sp.P) & 1u) || sp.P == l || (l >= 0 && ((dense >> l) & 1u))) return false;
+  sp.A = l >= 0 ? l : (sp.P == 0 ? 1 : 0);
+  sp.C = -1;
+  for (int q = 0; q < nd.nl; ++q)
+    if (q != sp.P && q != sp.A) sp.C = q;
+  sp.Da = nd.dims[sp.A];
+  sp.sA = nd.strides[sp.A];
+  sp.Dc = sp.C >= 0 ? nd.dims[sp.C] : 1;
+  sp.sC = sp.C >= 0 ? nd.strides[sp.C] : 0;
+  sp.dp = nd.dims[sp.P];
+  sp.sP = nd.strides[sp.P];
+  // exponentials read pairs of a row (even rows), projections read columns (odd rows: no bank
+  // conflicts)
+  sp.Cp = env ? (sp.Dc | 1) : sp.Dc + (sp.Dc & 1);
+  for (int pass = 0; pass < 2; ++pass) {
+    for (const Pair& pr : prs) {
+      if ((pr.d != nullptr) != (pass == 0)) continue;
+      for (int q = 0; q < (pr.s ? pr.s->nnz : 1); ++q) {
+        SiteJob& j = sp.job[sp.nj++];
+        j.type = pr.d ? (pr.d->leg == sp.A ? 0 : 1) : 2;
+        j.blk = pr.blk;
+        j.K = pr.d ? nd.dims[pr.d->leg] : 0;
+        j.mat = pr.d ? pr.d->mat - I.rega_off : 0;
+        j.nnz = pr.s ? pr.s->nnz : 0;
+        j.q = q;
+        j.sp = pr.s ? pr.s->sp - I.rega_off : 0;
+      }
+    }
+    if (pass == 0) sp.nd = sp.nj;
+  }
+  // the split with the fewest elements per CTA, fewest P indices per CTA among equals
+  int best = 1 << 30;
+  for (int sb = 1; sb <= sp.dp; ++sb) {
+    const int ns = (sp.dp + sb - 1) / sb;
+    if (ns > team) continue;
+    const int na0 = std::min(sp.Da, std::max(1, team / ns));
+    const int Ab = (sp.Da + na0 - 1) / na0;
+    if (Ab * sb < best) {
+      best = Ab * sb;
+      sp.sb = sb;
+      sp.ns = ns;
+      sp.Ab = Ab;
+      sp.na = (sp.Da + Ab - 1) / Ab;
+    }
+  }
+  // slices that each P range reads
+  for (int b = 0; b < sp.ns; ++b) {
+    for (int s = b * sp.sb; s < std::min(sp.dp, (b + 1) * sp.sb); ++s) {
+      sp.need[b] |= 1ull << s;
+      for (int j = 0; j < sp.nj; ++j) {
+        if (sp.job[j].nnz == 0) continue;
+        const long long at = I.rega_off + sp.job[j].sp + (long long)s * sp.job[j].nnz + sp.job[j].q;
+        const double2 v = C.pool_init[at];
+        if (v.x != 0.0 || v.y != 0.0) sp.need[b] |= 1ull << (int)C.pool_init[at + (long long)sp.dp * sp.job[j].nnz].x;
+      }
+    }
+    sp.max_sl = std::max(sp.max_sl, __builtin_popcountll(sp.need[b]));
+  }
+  // shared-memory layout
+  auto up = [](long long x) { return (x + 15) & ~15LL; };
+  long long off = up(sizeof(SitePlan));
+  sp.vals = (int)off;
+  off += (long long)sp.nj * sp.dp * vsize;
+  sp.cols = (int)off;
+  off = up(off + (long long)sp.nj * sp.dp * sizeof(int));
+  sp.mats = (int)off;
+  long long m = 0;
+  for (int j = 0; j < sp.nd; ++j) {
+    if (sp.job[j].q > 0) {  // the entries of one sparse factor share their matrix
+      sp.job[j].moff = sp.job[j - 1].moff;
+      continue;
+    }
+    sp.job[j].moff = (int)m;
+    m += sp.job[j].type == 0 ? ((sp.Ab * sp.Da + 1) & ~1) : sp.Dc * (sp.Dc + (sp.Dc & 1));
+  }
+  off = up(off + m * (long long)vsize);
+  sp.xs = (int)off;
+  off = up(off + (long long)sp.max_sl * sp.Da * sp.Cp * (long long)vsize);
+  sp.dbuf = (int)off;
+  const long long own = (long long)sp.Ab * sp.Dc * sp.sb;
+  off += sp.nd * own * (long long)vsize;
+  if (env) off += (1LL + I.nchan) * sp.sb * sp.Ab * sp.Cp * (long long)vsize;
+  off = up(off);
+  if (off > smem) return false;
+  sp.rest = (int)off;
+  *out = sp;
+  return true;
+}
+
+// Site plans of the whole program: one per distinct operation (the same node, leg and team recur
+// in a step), equal plans of different nodes shared.
+static void build_site_plans(ttns_tree* t, int grid, long long smem) {
+  Compiled& C = t->C;
+  t->sites.clear();
+  const size_t vsize = t->opt.precision == TTNS_FP64 ? sizeof(double2) : sizeof(float2);
+  std::unordered_map<unsigned long long, int> by_op;
+  std::unordered_multimap<unsigned long long, int> by_plan;
+  auto words = [](const SitePlan& sp, auto&& fn) {  // the parts in use
+    const char* b = reinterpret_cast<const char*>(&sp);
+    fn(b, offsetof(SitePlan, need) + sizeof(sp.need[0]) * sp.ns);
+    fn(b + offsetof(SitePlan, job), sizeof(SiteJob) * sp.nj);
+  };
+  for (Instr& I : C.prog) {
+    I.site = -1;
+    if (I.op != OP_FWD && I.op != OP_ENV) continue;
+    // a term list belongs to one node, operator and (environment updates) leg
+    const unsigned long long key = ((unsigned long long)I.terms << 2) | (I.op == OP_ENV ? 2u : 0u) | (I.team == TEAM_GRID);
+    const auto hit = by_op.find(key);
+    if (hit != by_op.end()) {
+      I.site = hit->second;
+      continue;
+    }
+    SitePlan sp;
+    if (site_plan(C, I, I.team == TEAM_GRID ? grid : t->cluster, vsize, smem, &sp)) {
+      unsigned long long h = 1469598103934665603ULL;
+      words(sp, [&](const char* b, size_t n) {
+        for (size_t k = 0; k + 4 <= n; k += 4) {
+          unsigned w;
+          std::memcpy(&w, b + k, 4);
+          h = (h ^ w) * 1099511628211ULL;
+        }
+      });
+      const auto range = by_plan.equal_range(h);
+      for (auto it = range.first; it != range.second && I.site < 0; ++it)
+        if (std::memcmp(&t->sites[it->second], &sp, sizeof(sp)) == 0) I.site = it->second;
+      if (I.site < 0) {
+        I.site = (int)t->sites.size();
+        t->sites.push_back(sp);
+        by_plan.emplace(h, I.site);
+      }
+    }
+    by_op.emplace(key, I.site);
+  }
+}
+
 static ttns_status device_init(ttns_tree* t) {
   Compiled& C = t->C;
   const ttns_options& o = t->opt;
@@ -370,7 +556,7 @@ static ttns_status device_init(ttns_tree* t) {
   t->cluster = o.cluster_ctas > 0 ? o.cluster_ctas : 16;
   if (t->cluster > 16) return fail(TTNS_E_INVALID, "cluster_ctas must be <= 16");
   int maxgrid = 0;
-  const long long smem_bytes = 200 * 1024;
+  const long long smem_bytes = 201 * 1024;  // with the kernel's static shared memory, all of an SM's 227 KB
   // the QR keeps three reduction buffers of 2 n^2 doubles (n <= TTNS_MAX_D) in it
   static_assert(3LL * 2 * TTNS_MAX_D * TTNS_MAX_D * 8 <= 200 * 1024, "QR reduction buffers exceed the shared memory");
   CUDA_TRY(max_grid_for(t->cluster, smem_bytes, &maxgrid));
@@ -395,6 +581,8 @@ static ttns_status device_init(ttns_tree* t) {
   if ((s = upload(t, &t->d_terms, C.terms)) != TTNS_OK) return s;
   if ((s = upload(t, &t->d_lists, C.lists)) != TTNS_OK) return s;
   if ((s = upload(t, &t->d_chans, C.chans)) != TTNS_OK) return s;
+  build_site_plans(t, grid, smem_bytes);
+  if ((s = upload(t, &t->d_sites, t->sites)) != TTNS_OK) return s;
   if ((s = upload(t, &t->d_prog, C.prog)) != TTNS_OK) return s;
   if ((s = upload(t, &t->d_trees, C.trees)) != TTNS_OK) return s;
   if ((s = dalloc(t, &t->ctl, 1)) != TTNS_OK) return s;
@@ -431,6 +619,7 @@ static ttns_status device_init(ttns_tree* t) {
   P.chans = t->d_chans;
   P.prog = t->d_prog;
   P.trees = t->d_trees;
+  P.sites = t->d_sites;
   P.n_trees = (int)C.trees.size();
   P.batched = t->batched ? 1 : 0;
   P.ctl = t->ctl;
@@ -1061,6 +1250,9 @@ extern "C" ttns_status ttns_grow_bonds(ttns_tree* t, const int* new_bond, int n_
   if (cudaMemcpy(t2->ctl, &hc, sizeof(Ctl), cudaMemcpyHostToDevice) != cudaSuccess)
     return abort_with(fail(TTNS_E_CUDA, "control block write failed"));
   if ((s = run_phase(t2, 3, "completion of grown bonds: ")) != TTNS_OK) return abort_with(s);
+  // the environment pass reads the tensors from the FP32 mirror
+  if (t2->pool32 && launch_mirror32(t2->pool, t2->pool32, t2->C.pool_size, t2->stream) != cudaSuccess)
+    return abort_with(fail(TTNS_E_CUDA, "mirror of the grown tree failed"));
   if ((s = run_phase(t2, 0, "environment pass after growth: ")) != TTNS_OK) return abort_with(s);
   t2->t_fs = t->t_fs;
   t2->launch_fallbacks += t->launch_fallbacks;

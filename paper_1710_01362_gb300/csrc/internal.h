@@ -75,6 +75,8 @@ struct Instr {
   int terms;       // index into the TermList table (FWD, ENV H-block, BOND)
   int chan_first;  // ENV: first channel Factor in the factor table
   int nchan;       // ENV: number of channel blocks
+  int site;        // FWD / ENV: index into the site plans (-1: none; see SitePlan)
+  unsigned adj;    // ENV: bit c: channel c's operator is the adjoint of channel c - 1's
   long long env_out;  // ENV: offset of the (1 + nchan) output blocks, each D x D
   int D;           // ENV / BOND / QR: dimension of the bond
   int D2;          // BOND: second dimension of the bond matrix
@@ -129,6 +131,8 @@ struct Ctl {
   unsigned pad1;
 };
 
+struct SitePlan;
+
 struct KernelParams {
   double2* pool;           // complex pool
   float2* pool32;          // FP32 mirror of the pool's operator data (mixed modes; else null):
@@ -139,6 +143,7 @@ struct KernelParams {
   const Factor* chans;
   const Instr* prog;
   const TreeDesc* trees;
+  const SitePlan* sites;
   int n_trees;
   int batched;             // 1: each cluster runs whole trees; 0: one tree, mixed teams
   Ctl* ctl;
@@ -169,6 +174,29 @@ struct KernelParams {
   long long smem_bytes;    // dynamic shared memory per CTA (operator matrices of one op)
   int cluster_resident;    // 1: small-node Krylov exponentials kept in the cluster's shared memory
   double qr_cutoff;        // relative null threshold of the QR
+};
+
+// Plan of an operation on a "site" tensor (site.cuh): legs, jobs, the split over the team and the
+// shared-memory layout.  Built on the host; offsets of operator data are relative to the
+// instruction's first operator region, so that equal sites share a plan.
+struct SiteJob {
+  int type;       // 0: dense on A, 1: dense on C, 2: sparse only
+  int blk;        // environment updates: output block
+  int moff, K;    // staged matrix (element offset) and its dimension
+  int nnz, q;     // row-sparse factor: entries per row (0: none) and the entry of this job
+  long long mat, sp;
+};
+constexpr int kSiteJobs = 48;
+struct SitePlan {
+  int A, C, P;                 // legs (C < 0: none)
+  int Da, Dc, dp, sA, sC, sP;  // dimensions and strides
+  int Cp;                      // padded row length of slices
+  int sb, ns, Ab, na;          // P indices and A rows per unit, units = ns * na
+  int nj, nd;                  // jobs, dense ones first
+  int max_sl;                  // largest number of slices that a unit reads
+  int vals, cols, mats, xs, dbuf, rest;  // byte offsets in the dynamic shared memory
+  unsigned long long need[TTNS_MAX_D];   // per P range: the slices that its units read
+  SiteJob job[kSiteJobs];
 };
 
 // One level (or a part of one) of the downward pass of bond densities: the nodes, and the

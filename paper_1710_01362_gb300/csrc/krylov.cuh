@@ -211,7 +211,7 @@ __device__ __noinline__ void texp_warp(const double* a, const double* b, int m, 
 // Convergence of step m: beta_m |e_m^T exp(-i s T_m) e_0| <= tol.  Component m of the expansion
 // has no contribution from orders below m - 1, and those above fall off as (z / 2)^n / n!, so
 // every term and the sum keep FP32's relative accuracy however small the component is: the
-// check runs in FP32 (an FP64 expansion takes 4 us and more on one warp); wide spectra (z > 16),
+// check runs in FP32 (an FP64 expansion takes 4 us and more on one warp); wide spectra (z > 28),
 // where many orders below m carry weight, take the FP64 expansion.  No margin: one step more or
 // less changes what is left below the tolerance, and the QR's null decisions can amplify that.
 __device__ __noinline__ bool krylov_small(const KrylovShared& ks, int m, double s, double tol, double* ure,
@@ -221,14 +221,14 @@ __device__ __noinline__ bool krylov_small(const KrylovShared& ks, int m, double 
   ChebSetup cs = cheb_setup(ks.alpha, ks.beta, m, fabsf((float)s));
   *nonfinite = false;
   float um;
-  if (cs.z <= 16.f) {
+  if (cs.z <= 28.f) {
     cheb_order(cs, cs.z);
     const int K = min(64, cs.K + 4);
     const float y = -0.25f * cs.z * cs.z;
     float h0 = 1.f, h1 = 1.f;
     for (int j = 8 + (int)(2.f * cs.z); j >= 1; --j) {  // J_n = (z/2)^n / n! sum_j y^j n! / (j! (n+j)!)
-      h0 = fmaf(h0 * y, 1.f / (float)(j * (j + lane)), 1.f);
-      h1 = fmaf(h1 * y, 1.f / (float)(j * (j + lane + 32)), 1.f);
+      h0 = fmaf(h0 * y, __fdividef(1.f, (float)(j * (j + lane))), 1.f);
+      h1 = fmaf(h1 * y, __fdividef(1.f, (float)(j * (j + lane + 32))), 1.f);
     }
     const float J0 = cs.p0 * h0, J1 = cs.p1 * h1;
     const float ri = cs.R > 0.f ? 2.f / cs.R : 0.f;
@@ -666,6 +666,33 @@ __device__ __forceinline__ double orth_slices(Team& tm, KF&& Ks, int n_own, int 
   return nrm;
 }
 
+// y = beta0 sum_k u_k q_k into the own part of K_0; returns this thread's share of |y|^2
+template <typename KF>
+__device__ __forceinline__ double krylov_combine(const KrylovShared& ks, KF&& Ks, int n_own, int m) {
+  double ny = 0.0;
+  for (int e = threadIdx.x; e < n_own; e += NT) {
+    double yr = 0.0, yi = 0.0, zr = 0.0, zi = 0.0;  // two chains
+    int k = 0;
+    for (; k + 1 < m; k += 2) {
+      const double2 q = Ks(k)[e], p = Ks(k + 1)[e];
+      yr = fma(ks.ure[k], q.x, fma(-ks.uim[k], q.y, yr));
+      yi = fma(ks.ure[k], q.y, fma(ks.uim[k], q.x, yi));
+      zr = fma(ks.ure[k + 1], p.x, fma(-ks.uim[k + 1], p.y, zr));
+      zi = fma(ks.ure[k + 1], p.y, fma(ks.uim[k + 1], p.x, zi));
+    }
+    if (k < m) {
+      const double2 q = Ks(k)[e];
+      yr = fma(ks.ure[k], q.x, fma(-ks.uim[k], q.y, yr));
+      yi = fma(ks.ure[k], q.y, fma(ks.uim[k], q.x, yi));
+    }
+    yr += zr;
+    yi += zi;
+    Ks(0)[e] = make_double2(yr, yi);
+    ny = fma(yr, yr, fma(yi, yi, ny));
+  }
+  return ny;
+}
+
 template <typename T>
 __device__ __noinline__ bool op_expm_cluster(const KernelParams& P, Team& tm, const Instr& I, double2* work,
                                              double tau) {
@@ -739,7 +766,7 @@ __device__ __noinline__ bool op_expm_cluster(const KernelParams& P, Team& tm, co
       v[0] = fma(a.x, a.x, fma(a.y, a.y, v[0]));
       publish(e0 + e, cvt<T>(a));
     }
-    team_reduce<1>(tm, v, [&](const double* t) { krylov_begin(ks, t[0]); });
+    team_reduce<1>(tm, v, [&](const double* t) { krylov_begin(ks, t[0]); }, n_own);
     pc.lap(P.ctl, 6);
     const double beta0 = ks.beta0;
     if (!(beta0 > 0.0)) {
@@ -809,9 +836,9 @@ __device__ __noinline__ bool op_expm_cluster(const KernelParams& P, Team& tm, co
         W[e] = make_double2(wr, wi);
       }
       if constexpr (kShadow)
-        team_reduce<3>(tm, part, [&](const double* t) { krylov_alpha(ks, j, t[0], t[1], t[2]); });
+        team_reduce<3>(tm, part, [&](const double* t) { krylov_alpha(ks, j, t[0], t[1], t[2]); }, n_own);
       else
-        team_reduce<1>(tm, part, [&](const double* t) { krylov_alpha(ks, j, t[0]); });
+        team_reduce<1>(tm, part, [&](const double* t) { krylov_alpha(ks, j, t[0]); }, n_own);
       pc.lap(P.ctl, 2);
       const double ca = ks.ca;  // alpha_j scale_j
       if (kShadow && ks.fused && threadIdx.x == NT - 32) krylov_norm(ks, j, ks.b2, s_rem, P.tol, mmax);
@@ -837,7 +864,7 @@ __device__ __noinline__ bool op_expm_cluster(const KernelParams& P, Team& tm, co
       if (fused)
         team_sync(tm);  // K_{j+1} is complete on every CTA before the next application
       else
-        team_reduce<1>(tm, nrm, [&](const double* t) { krylov_norm(ks, j, t[0], s_rem, P.tol, mmax); });
+        team_reduce<1>(tm, nrm, [&](const double* t) { krylov_norm(ks, j, t[0], s_rem, P.tol, mmax); }, n_own);
       pc.lap(P.ctl, 3);
       m = j + 1;
       if (ks.check) {
@@ -854,32 +881,11 @@ __device__ __noinline__ bool op_expm_cluster(const KernelParams& P, Team& tm, co
     __syncthreads();
     const double s_done = ks.s_done;
     pc.lap(P.ctl, 4);
-    // y = beta0 sum_k u_k q_k into the own slice of K_0
-    double ny[1] = {0.0};
-    for (int e = threadIdx.x; e < n_own; e += NT) {
-      double yr = 0.0, yi = 0.0, zr = 0.0, zi = 0.0;  // two chains
-      int k = 0;
-      for (; k + 1 < m; k += 2) {
-        const double2 q = Ks(k)[e], p = Ks(k + 1)[e];
-        yr = fma(ks.ure[k], q.x, fma(-ks.uim[k], q.y, yr));
-        yi = fma(ks.ure[k], q.y, fma(ks.uim[k], q.x, yi));
-        zr = fma(ks.ure[k + 1], p.x, fma(-ks.uim[k + 1], p.y, zr));
-        zi = fma(ks.ure[k + 1], p.y, fma(ks.uim[k + 1], p.x, zi));
-      }
-      if (k < m) {
-        const double2 q = Ks(k)[e];
-        yr = fma(ks.ure[k], q.x, fma(-ks.uim[k], q.y, yr));
-        yi = fma(ks.ure[k], q.y, fma(ks.uim[k], q.x, yi));
-      }
-      yr += zr;
-      yi += zi;
-      Ks(0)[e] = make_double2(yr, yi);
-      if constexpr (kShadow) ny[0] = fma(yr, yr, fma(yi, yi, ny[0]));
-    }
+    double ny[1] = {krylov_combine(ks, Ks, n_own, m)};
     if constexpr (kShadow) {
       // the exact exponential is unitary; FP32-class contractions leave the basis orthonormal
       // only to ~1e-7, so the norm is restored to the input's
-      team_reduce<1>(tm, ny, [&](const double* t) { ks.ratio = t[0] > 0.0 ? ks.beta0 / sqrt(t[0]) : 1.0; });
+      team_reduce<1>(tm, ny, [&](const double* t) { ks.ratio = t[0] > 0.0 ? ks.beta0 / sqrt(t[0]) : 1.0; }, n_own);
       const double ratio = ks.ratio;
       if (fabs(ratio - 1.0) < 1e-3)
         for (int e = threadIdx.x; e < n_own; e += NT) {

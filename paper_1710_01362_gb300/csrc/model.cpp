@@ -672,6 +672,18 @@ struct TreeCompiler {
     I.D = C.nodes[I.node].dims[I.leg];
     C.prog.push_back(I);
   }
+  // b's operators are exactly the adjoints of a's, on the same nodes
+  static bool adjoint_pair(const Coupling& a, const Coupling& b) {
+    auto adj = [](const std::vector<cplx>& x, const std::vector<cplx>& y) {
+      const size_t n = (size_t)std::lround(std::sqrt((double)x.size()));
+      if (x.size() != y.size()) return false;
+      for (size_t i = 0; i < n; ++i)
+        for (size_t j = 0; j < n; ++j)
+          if (y[i * n + j] != std::conj(x[j * n + i])) return false;
+      return true;
+    };
+    return a.va == b.va && a.vb == b.vb && adj(a.opa, b.opa) && adj(a.opb, b.opb);
+  }
   void emit_env(int u, int v) {
     auto key = std::make_pair(u, v);
     auto it = envh_list.find(key);
@@ -700,6 +712,9 @@ struct TreeCompiler {
     I.terms = li;
     I.chan_first = env_chan[key].first;
     I.nchan = env_chan[key].second;
+    // the two halves of a hopping term follow each other: the second block is the first's adjoint
+    for (int c = 1; c < I.nchan && c < 32; ++c)
+      if (!((I.adj >> (c - 1)) & 1u) && adjoint_pair(t.coups[E.chans[c - 1]], t.coups[E.chans[c]])) I.adj |= 1u << c;
     I.env_out = E.off;
     I.D = E.D;
     I.flops = list_flops(li, C.nodes[I.node]) + 8.0 * C.nodes[I.node].size * E.D * (1 + E.chans.size());

@@ -627,7 +627,11 @@ __device__ __noinline__ void op_qr(const KernelParams& P, Team& tm, const Instr&
       o_r.init(A::zero());
       o_i.init(A::zero());
       q_cmac<A>(o_r, o_i, A::c(qr, qi), A::cfrom(qs.ph[c]));
-      Ag[qr_addr(nd, l, r, c)] = A::cto(A::c(o_r.val(), o_i.val()));
+      const long long at = qr_addr(nd, l, r, c);
+      const E v = A::c(o_r.val(), o_i.val());
+      Ag[at] = A::cto(v);
+      // the mixed modes' environment updates read Q from the FP32 mirror (the heads of v)
+      if constexpr (std::is_same<A, QrDs>::value) P.pool32[nd.off + at] = make_float2(A::re(v).x, A::im(v).x);
     };
     put(c0, q0r.val(), q0i.val());
     if (c1 > c0) put(c1, q1r.val(), q1i.val());

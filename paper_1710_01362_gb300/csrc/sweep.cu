@@ -216,18 +216,21 @@ __device__ __forceinline__ double warp_reduce_t(double* v) {
 // 20 cycles whatever its lanes do).  Cluster teams push each CTA's totals into every peer's
 // shared memory before the cluster barrier, so that after it the sums come from local shared
 // memory; the grid team goes through global memory.  `fin` runs on thread 0 with the totals
-// before the last block barrier: scalars derived from them are computed once and read from
+// before the last block barrier (`nact`: the first threads that hold values; the others' are not
+// read): scalars derived from them are computed once and read from
 // shared memory (a square root that all eight warps repeat costs 2500 cycles).
 static_assert(NT == 256, "team_reduce assumes 256 threads per CTA");
 __shared__ double s_all[4][NT];
 __shared__ double s_recv[2][16][4];  // [parity][source rank][value] (cluster teams, <= 16 CTAs)
 template <int NV>
-__device__ __noinline__ void team_total(Team& tm, const double* v, double* tot) {  // totals on warp 0
+__device__ __noinline__ void team_total(Team& tm, const double* v, double* tot, int nact) {  // totals on warp 0
   static_assert(NV <= 4, "up to four values");
   constexpr int NB = NV == 1 ? 1 : (NV == 2 ? 2 : 4);  // values of the butterfly
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rows = (min(nact, NT) + 31) >> 5;  // warps with values: four or all of them are added
+  if (warp < (rows <= 4 ? 4 : 8))
 #pragma unroll
-  for (int i = 0; i < NV; ++i) s_all[i][threadIdx.x] = v[i];
+    for (int i = 0; i < NV; ++i) s_all[i][threadIdx.x] = v[i];
   __syncthreads();
   double t[NB];
 #pragma unroll
@@ -236,8 +239,13 @@ __device__ __noinline__ void team_total(Team& tm, const double* v, double* tot) 
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
       const double* a = s_all[i];
-      t[i] = ((a[lane] + a[lane + 32]) + (a[lane + 64] + a[lane + 96])) +
-             ((a[lane + 128] + a[lane + 160]) + (a[lane + 192] + a[lane + 224]));
+      if (rows <= 1)
+        t[i] = a[lane];
+      else if (rows <= 2)
+        t[i] = a[lane] + a[lane + 32];
+      else
+        t[i] = (a[lane] + a[lane + 32]) + (a[lane + 64] + a[lane + 96]);
+      if (rows > 4) t[i] += (a[lane + 128] + a[lane + 160]) + (a[lane + 192] + a[lane + 224]);
     }
     const double r = warp_reduce_t<NB>(t);
 #pragma unroll
@@ -280,9 +288,9 @@ __device__ __noinline__ void team_total(Team& tm, const double* v, double* tot) 
   tm.parity ^= 1;
 }
 template <int NV, typename F>
-__device__ __forceinline__ void team_reduce(Team& tm, const double* v, F&& fin) {
+__device__ __forceinline__ void team_reduce(Team& tm, const double* v, F&& fin, int nact = NT) {
   double tot[NV];
-  team_total<NV>(tm, v, tot);
+  team_total<NV>(tm, v, tot, nact);
   if (threadIdx.x == 0) fin(tot);
   __syncthreads();
 }
@@ -1469,64 +1477,14 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
 
 #include "qr.cuh"
 
-// ------------------------------------------------------------------ absorb
-// A_u <- R applied on leg I.leg (FP64), through a temporary
-__device__ __noinline__ void op_absorb(const KernelParams& P, Team& tm, const Instr& I, double2* work) {
-  const NodeDesc nd = P.nodes[I.node];
-  const long long N = nd.size;
-  double2* A = P.pool + nd.off;
-  const double2* R = P.pool + P.trees[I.tree].bond_off;
-  const int l = I.leg;
-  for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
-    LegPos lp = leg_pos(nd, l, idx);
-    auto a = mode_dot<double>(R + (long long)lp.i * nd.dims[l], nd.dims[l], A, lp.base, nd.strides[l]);
-    work[idx] = a;
-  }
-  team_sync(tm);
-  for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) A[idx] = work[idx];
-  team_sync(tm);
-}
-
-// A_u <- R applied on leg I.leg (the gauge absorb of the mixed modes) in double-single: the
-// tensor is converted once into the workspace, R into shared memory, every element is a
-// compensated dot of length dims[leg], and the result is written back in FP64.
-__device__ __noinline__ void op_absorb_ds(const KernelParams& P, Team& tm, const Instr& I, double2* work) {
-  const NodeDesc nd = P.nodes[I.node];
-  const long long N = nd.size;
-  double2* A = P.pool + nd.off;
-  const double2* R = P.pool + P.trees[I.tree].bond_off;
-  const int l = I.leg;
-  const int D = nd.dims[l];
-  const int st = nd.strides[l];
-  float4* Ad = reinterpret_cast<float4*>(work);
-  float4* Rd = reinterpret_cast<float4*>(dyn_smem);  // D x D <= 64 KB
-  for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) Ad[idx] = ds_cfrom(A[idx]);
-  for (int k = threadIdx.x; k < D * D; k += NT) Rd[k] = ds_cfrom(R[k]);
-  team_sync(tm);
-  for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
-    const LegPos lp = leg_pos(nd, l, idx);
-    const float4* row = Rd + lp.i * D;
-    const float4* xp = Ad + lp.base;
-    DsAcc ar0, ai0, ar1, ai1;
-    ar0.init(make_float2(0.f, 0.f));
-    ai0.init(make_float2(0.f, 0.f));
-    ar1.init(make_float2(0.f, 0.f));
-    ai1.init(make_float2(0.f, 0.f));
-    int k = 0;
-    for (; k + 1 < D; k += 2) {
-      ds_cmac(ar0, ai0, row[k], xp[(long long)k * st]);
-      ds_cmac(ar1, ai1, row[k + 1], xp[(long long)(k + 1) * st]);
-    }
-    if (k < D) ds_cmac(ar0, ai0, row[k], xp[(long long)k * st]);
-    const float2 r = ds_add(ar0.val(), ar1.val()), i = ds_add(ai0.val(), ai1.val());
-    A[idx] = make_double2(ds_to(r), ds_to(i));
-  }
-  team_sync(tm);
-}
+#include "absorb.cuh"
+#include "site.cuh"
 
 // ------------------------------------------------------------------ environment update
 // env(u -> v): block 0 = Q^H (H-terms of u without v) Q, block 1+b = Q^H (channel factor b) Q,
-// contracted over every leg of Q except the leg toward v.
+// contracted over every leg of Q except the leg toward v.  This form takes the tensors that are
+// not sites (ER nodes, roots of several chains, OBB sites): results of all rows in global memory,
+// every output value summed over all rows by one CTA.
 template <typename T>
 __device__ __noinline__ void op_env(const KernelParams& P, Team& tm, const Instr& I, double2* work) {
   const NodeDesc nd = P.nodes[I.node];
@@ -1703,7 +1661,8 @@ __device__ void exec_op(const KernelParams& P, Team& tm, const Instr& I, double2
   switch (I.op) {
     case OP_FWD:
     case OP_BOND:
-      if (!(tm.kind == TEAM_CLUSTER && P.cluster_resident && op_expm_cluster<T>(P, tm, I, work, tau)))
+      if (!op_expm_site<T>(P, tm, I, work, tau) &&
+          !(tm.kind == TEAM_CLUSTER && P.cluster_resident && op_expm_cluster<T>(P, tm, I, work, tau)))
         op_expm<T>(P, tm, I, work, tau);
       break;
     case OP_QR:
@@ -1713,19 +1672,41 @@ __device__ void exec_op(const KernelParams& P, Team& tm, const Instr& I, double2
         op_qr<QrDs>(P, tm, I, work);
       break;
     case OP_ENV:
-      op_env<T>(P, tm, I, work);
+      if (!op_env_site<T>(P, tm, I)) op_env<T>(P, tm, I, work);
       break;
     case OP_ABSORB:
       if constexpr (std::is_same<T, double>::value)
-        op_absorb(P, tm, I, work);
+        op_absorb<QrF64>(P, tm, I);
       else
-        op_absorb_ds(P, tm, I, work);
+        op_absorb<QrDs>(P, tm, I);
       break;
     case OP_RECORD:
       op_record(P, tm, I, P.traj_count + I.tree);
       break;
   }
 }
+
+// The current instruction in shared memory; the next one's words are loaded into registers while
+// it runs, so that no operation starts with a chain of global loads for its own record.
+__shared__ Instr s_instr;
+struct InstrFeed {
+  static constexpr int kWords = (int)(sizeof(Instr) / 4);
+  static_assert(kWords <= NT && sizeof(Instr) % 4 == 0, "one word per thread");
+  const unsigned* p;
+  unsigned w;
+  __device__ InstrFeed(const Instr* prog) : p(reinterpret_cast<const unsigned*>(prog)), w(0) {
+    if (threadIdx.x < kWords) w = p[threadIdx.x];
+  }
+  __device__ void next(bool more) {
+    __syncthreads();  // the last instruction is done
+    if (threadIdx.x < kWords) {
+      reinterpret_cast<unsigned*>(&s_instr)[threadIdx.x] = w;
+      p += kWords;
+      if (more) w = p[threadIdx.x];
+    }
+    __syncthreads();
+  }
+};
 
 template <typename T>
 __device__ void run(const KernelParams& P, int phase) {
@@ -1751,8 +1732,10 @@ __device__ void run(const KernelParams& P, int phase) {
       const int count = phase == 0 ? td.init_count : (phase == 2 ? td.obs_count : (phase == 3 ? td.grow_count : td.prog_count));
       const int nst = phase == 1 ? P.n_steps : 1;
       for (int s = 0; s < nst; ++s) {
+        InstrFeed feed(P.prog + first);
         for (int k = 0; k < count; ++k) {
-          exec<T>(P, ct, P.prog[first + k], cwork);
+          feed.next(k + 1 < count);
+          exec<T>(P, ct, s_instr, cwork);
         }
       }
     }
@@ -1774,8 +1757,10 @@ __device__ void run(const KernelParams& P, int phase) {
   const int nst = phase == 1 ? P.n_steps : 1;
   int prev = TEAM_GRID;
   for (int s = 0; s < nst; ++s) {
+    InstrFeed feed(P.prog + first);
     for (int k = 0; k < count; ++k) {
-      const Instr& I = P.prog[first + k];
+      feed.next(k + 1 < count);
+      const Instr& I = s_instr;
       if (I.team == TEAM_GRID) {
         if (prev == TEAM_CLUSTER) grid_sync(P.ctl, P.spin_limit);
         exec<T>(P, gt, I, P.work);
