@@ -5,7 +5,7 @@
 // them, so the product is done in place: no second copy of the tensor and no barrier between
 // reading and writing.  The fibres are converted once into shared memory (k-major), R too, and
 // few outputs per CTA are split over two or four lanes each.  (40 x 40 x 20 tensors of the ER
-// tree on the whole grid: 24 us per absorb with a converted global copy before, @ABS now.)
+// tree on the whole grid: 24 us per absorb with a converted global copy before, 15 us now.)
 template <typename A>
 __device__ __noinline__ void op_absorb(const KernelParams& P, Team& tm, const Instr& I) {
   using E = typename A::E;

@@ -378,6 +378,7 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
     const Factor *d, *s;
   };
   std::vector<Pair> prs;
+  prs.reserve(L.count + 16);
   auto add = [&](int blk, const Factor* a, const Factor* b) {
     Pair pr{blk, nullptr, nullptr};
     for (const Factor* f : {a, b}) {
@@ -415,15 +416,6 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
   sp.C = -1;
   for (int q = 0; q < nd.nl; ++q)
     if (q != sp.P && q != sp.A) sp.C = q;
-  sp.Da = nd.dims[sp.A];
-  sp.sA = nd.strides[sp.A];
-  sp.Dc = sp.C >= 0 ? nd.dims[sp.C] : 1;
-  sp.sC = sp.C >= 0 ? nd.strides[sp.C] : 0;
-  sp.dp = nd.dims[sp.P];
-  sp.sP = nd.strides[sp.P];
-  // exponentials read pairs of a row (even rows), projections read columns (odd rows: no bank
-  // conflicts)
-  sp.Cp = env ? (sp.Dc | 1) : sp.Dc + (sp.Dc & 1);
   for (int pass = 0; pass < 2; ++pass) {
     for (const Pair& pr : prs) {
       if ((pr.d != nullptr) != (pass == 0)) continue;
@@ -440,6 +432,15 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
     }
     if (pass == 0) sp.nd = sp.nj;
   }
+  sp.Da = nd.dims[sp.A];
+  sp.sA = nd.strides[sp.A];
+  sp.Dc = sp.C >= 0 ? nd.dims[sp.C] : 1;
+  sp.sC = sp.C >= 0 ? nd.strides[sp.C] : 0;
+  sp.dp = nd.dims[sp.P];
+  sp.sP = nd.strides[sp.P];
+  // exponentials read pairs of a row (even rows), projections read columns (odd rows: no bank
+  // conflicts)
+  sp.Cp = env ? (sp.Dc | 1) : sp.Dc + (sp.Dc & 1);
   // the split with the fewest elements per CTA, fewest P indices per CTA among equals
   int best = 1 << 30;
   for (int sb = 1; sb <= sp.dp; ++sb) {
@@ -505,7 +506,8 @@ static void build_site_plans(ttns_tree* t, int grid, long long smem) {
   Compiled& C = t->C;
   t->sites.clear();
   const size_t vsize = t->opt.precision == TTNS_FP64 ? sizeof(double2) : sizeof(float2);
-  std::unordered_map<unsigned long long, int> by_op;
+  constexpr int kNone = -2;
+  std::vector<int> by_op(C.lists.size() * 4, kNone);
   std::unordered_multimap<unsigned long long, int> by_plan;
   auto words = [](const SitePlan& sp, auto&& fn) {  // the parts in use
     const char* b = reinterpret_cast<const char*>(&sp);
@@ -516,20 +518,20 @@ static void build_site_plans(ttns_tree* t, int grid, long long smem) {
     I.site = -1;
     if (I.op != OP_FWD && I.op != OP_ENV) continue;
     // a term list belongs to one node, operator and (environment updates) leg
-    const unsigned long long key = ((unsigned long long)I.terms << 2) | (I.op == OP_ENV ? 2u : 0u) | (I.team == TEAM_GRID);
-    const auto hit = by_op.find(key);
-    if (hit != by_op.end()) {
-      I.site = hit->second;
+    int& known = by_op[4 * (size_t)I.terms + (I.op == OP_ENV ? 2 : 0) + (I.team == TEAM_GRID ? 1 : 0)];
+    if (known != kNone) {
+      I.site = known;
       continue;
     }
     SitePlan sp;
     if (site_plan(C, I, I.team == TEAM_GRID ? grid : t->cluster, vsize, smem, &sp)) {
       unsigned long long h = 1469598103934665603ULL;
       words(sp, [&](const char* b, size_t n) {
-        for (size_t k = 0; k + 4 <= n; k += 4) {
-          unsigned w;
-          std::memcpy(&w, b + k, 4);
+        for (size_t k = 0; k + 8 <= n; k += 8) {
+          unsigned long long w;
+          std::memcpy(&w, b + k, 8);
           h = (h ^ w) * 1099511628211ULL;
+          h ^= h >> 29;
         }
       });
       const auto range = by_plan.equal_range(h);
@@ -541,7 +543,7 @@ static void build_site_plans(ttns_tree* t, int grid, long long smem) {
         by_plan.emplace(h, I.site);
       }
     }
-    by_op.emplace(key, I.site);
+    known = I.site;
   }
 }
 
@@ -1245,7 +1247,6 @@ extern "C" ttns_status ttns_grow_bonds(ttns_tree* t, const int* new_bond, int n_
   if (cudaMemcpy(&hc, t->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost) != cudaSuccess)
     return abort_with(fail(TTNS_E_CUDA, "control block read failed"));
   hc.bar_count = 0;
-  hc.bar_gen = 0;
   hc.status = hc.err_where = hc.err_node = 0;
   if (cudaMemcpy(t2->ctl, &hc, sizeof(Ctl), cudaMemcpyHostToDevice) != cudaSuccess)
     return abort_with(fail(TTNS_E_CUDA, "control block write failed"));
@@ -1523,7 +1524,6 @@ ttns_status read_state(ttns_tree* t, FILE* f) {
   // the tensors are not validated here: a non-finite entry is reported by the next step
   // (TTNS_E_NONFINITE from the Krylov norm)
   h.bar_count = 0;
-  h.bar_gen = 0;
   h.status = 0;
   h.err_where = 0;
   h.err_node = 0;

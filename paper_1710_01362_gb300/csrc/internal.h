@@ -112,8 +112,7 @@ struct TreeDesc {
 
 // Device-side control block (status word, barrier, counters).
 struct Ctl {
-  unsigned bar_count;
-  unsigned bar_gen;
+  unsigned long long bar_count;  // arrivals of all clusters at all grid barriers
   int status;          // ttns_status of the device
   int pad0;
   unsigned long long krylov_iters;

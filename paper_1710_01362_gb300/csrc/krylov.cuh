@@ -231,7 +231,7 @@ __device__ __noinline__ bool krylov_small(const KrylovShared& ks, int m, double 
       h1 = fmaf(h1 * y, __fdividef(1.f, (float)(j * (j + lane + 32))), 1.f);
     }
     const float J0 = cs.p0 * h0, J1 = cs.p1 * h1;
-    const float ri = cs.R > 0.f ? 2.f / cs.R : 0.f;
+    const float ri = cs.R > 1e-30f ? 2.f / cs.R : 0.f;  // (a smaller radius is zero: its reciprocal overflows)
     const float dk = lane < m ? ri * (float)(ks.alpha[lane] - (double)cs.c) : 0.f;
     const float ek = (lane < m && lane > 0) ? ri * (float)ks.beta[lane] : 0.f;
     const float fk = lane + 1 < m ? ri * (float)ks.beta[lane + 1] : 0.f;
@@ -415,6 +415,7 @@ struct PhaseClock {
 // owner.
 struct ClTerm {
   int dD, dst, dl, doff;            // dense factor: dimension (0: none), stride, leg, staged position of row 0
+  int dr;                           // staged row length, odd: lanes on different rows read different banks
   int r0, nr;                       // staged rows
   int snnz, sD, sst, sl, soff;      // row-sparse factor: entries per row (0: none), ...
   int xo;                           // input: offset from xs (0, or a first factor's result)
@@ -462,7 +463,7 @@ __device__ __forceinline__ typename C2<T>::t cl_term(const ClTerm& c, const type
   using V = typename C2<T>::t;
   const V* x = xs + c.xo;
   const int i = (int)(pk >> (8 * c.dl)) & 255;
-  const V* row = sm + c.doff + i * c.dD;
+  const V* row = sm + c.doff + i * c.dr;
   if (c.snnz == 0) return dot_at<T>(row, c.dD, x + (e - i * c.dst), c.dst);
   const int is = (int)(pk >> (8 * c.sl)) & 255;
   const V* vals = sm + c.soff + is * c.snnz;
@@ -522,6 +523,7 @@ __device__ void cl_plan(const KernelParams& P, const NodeDesc& nd, const TermLis
         c.sp = f.sp;
       } else {
         c.dD = nd.dims[f.leg];
+        c.dr = c.dD | 1;
         c.dst = nd.strides[f.leg];
         c.dl = f.leg;
         c.dmat = f.mat;
@@ -561,8 +563,8 @@ __device__ void cl_plan(const KernelParams& P, const NodeDesc& nd, const TermLis
           c.r0 = c.hi > c.lo ? c.lo / c.dst : 0;
           c.nr = c.hi > c.lo ? (c.hi - 1) / c.dst - c.r0 + 1 : 0;
         }
-        c.doff = (int)m - c.r0 * c.dD;
-        m += (long long)rows * c.dD;
+        c.doff = (int)m - c.r0 * c.dr;
+        m += (long long)rows * c.dr;
       }
       if (c.snnz) {
         c.soff = (int)m;
@@ -589,18 +591,23 @@ template <typename T>
 __device__ void cl_stage(const KernelParams& P, const ClTerm* ct, int n, typename C2<T>::t* sm) {
   using V = typename C2<T>::t;
   const V* src = ops<T>(P);
-  auto copy = [&](V* d, const V* s, int cnt) {
-    for (int k = threadIdx.x; k < cnt; k += NT) {
-      if constexpr (sizeof(V) == 16)
-        cp_async16(d + k, s + k);
-      else
-        cp_async8(d + k, s + k);
-    }
+  auto cp = [&](V* d, const V* s) {
+    if constexpr (sizeof(V) == 16)
+      cp_async16(d, s);
+    else
+      cp_async8(d, s);
   };
   for (int t = 0; t < n; ++t) {
     const ClTerm& c = ct[t];
-    if (c.dD) copy(sm + c.doff + c.r0 * c.dD, src + c.dmat + (long long)c.r0 * c.dD, c.nr * c.dD);
-    if (c.snnz) copy(sm + c.soff, src + c.sp, 2 * c.sD * c.snnz);
+    if (c.dD) {
+      V* d = sm + c.doff + c.r0 * c.dr;
+      const V* s = src + c.dmat + (long long)c.r0 * c.dD;
+      const int pad = c.dr - c.dD;
+      const float inv = 1.0f / (float)c.dD;
+      for (int k = threadIdx.x; k < c.nr * c.dD; k += NT) cp(d + k + pad * fdivu(k, c.dD, inv), s + k);
+    }
+    if (c.snnz)
+      for (int k = threadIdx.x; k < 2 * c.sD * c.snnz; k += NT) cp(sm + c.soff + k, src + c.sp + k);
   }
   cp_async_wait_all();
 }

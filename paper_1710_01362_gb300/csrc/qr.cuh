@@ -18,7 +18,7 @@
 //   * everything after the column loop works on the active reflectors only, and Z of the
 //     compact form comes from one triangular solve (below) instead of T and T V^H.
 // Measured on the 800 x 40 tensors of the 8 x 60 ER tree (double-single, one 16-CTA cluster,
-// early in the run): 249 us per QR before, 47 us now; FP64: 354 and 70 us.
+// early in the run): 249 us per QR before, 41 us now; FP64: 354 and 65 us.
 //
 // The double-single arithmetic issues FP32 operations at about 80 times this part's FP64 rate;
 // it keeps every sum and product to about 2^-44 relative, far below the FP32-class error of the
@@ -169,7 +169,7 @@ struct QRShared {
   double2 ph[TTNS_MAX_D];
   int act[TTNS_MAX_D];       // active columns, ascending
   int na, next;
-  double tau;
+  double tau, dropped;
   double red[NWARP];
 };
 __shared__ QRShared s_qs;
@@ -207,7 +207,7 @@ __device__ __noinline__ void op_qr(const KernelParams& P, Team& tm, const Instr&
   const float inv_nr = nr > 0 ? 1.0f / (float)nr : 0.0f;
   // shared memory: two partial buffers and the sums (PB scalars each), the own rows of the
   // workspace (column-major, `chunk` rows per column) and Z when they fit, else global memory
-  const int PB = max(2 * n * n, 5 * n + 4);
+  const int PB = (max(2 * n * n, 5 * n + 4) + 1) & ~1;  // (even: the buffers also hold 16-byte elements)
   S* red[2] = {reinterpret_cast<S*>(dyn_smem), reinterpret_cast<S*>(dyn_smem) + PB};
   S* redo = red[1] + PB;
   int rp = 0;
@@ -228,13 +228,24 @@ __device__ __noinline__ void op_qr(const KernelParams& P, Team& tm, const Instr&
   // copy into the workspace; the Frobenius norm sets the null threshold
   Acc fro;
   fro.init(A::zero());
-  for (int idx = threadIdx.x; idx < n * nr; idx += NT) {
-    const int c = fdivu(idx, nr, inv_nr);
-    const int r = rb + (idx - c * nr);
-    const E a = A::cfrom(Ag[qr_addr(nd, l, r, c)]);
-    WA(c, r) = a;
-    fro.mac(A::re(a), A::re(a));
-    fro.mac(A::im(a), A::im(a));
+  for (int idx0 = threadIdx.x; idx0 < n * nr; idx0 += 4 * NT) {  // four loads in flight per thread
+    double2 g[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int idx = min(idx0 + u * NT, n * nr - 1);
+      const int c = fdivu(idx, nr, inv_nr);
+      g[u] = Ag[qr_addr(nd, l, rb + (idx - c * nr), c)];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int idx = idx0 + u * NT;
+      if (idx >= n * nr) break;
+      const int c = fdivu(idx, nr, inv_nr);
+      const E a = A::cfrom(g[u]);
+      WA(c, rb + (idx - c * nr)) = a;
+      fro.mac(A::re(a), A::re(a));
+      fro.mac(A::im(a), A::im(a));
+    }
   }
   __syncthreads();
   // This CTA's partials for column jj over its rows r > jj, for the columns c = jj .. n - 1:
@@ -352,6 +363,7 @@ __device__ __noinline__ void op_qr(const KernelParams& P, Team& tm, const Instr&
       for (int w = 1; w < NWARP; ++w) sum = A::add(sum, s_fro[w]);
       mine[4 * n] = sum;
       qs.na = 0;
+      qs.dropped = 0.0;
     }
     q_team_reduce<A>(tm, mine, redo, 4 * n + 1);
   }
@@ -370,6 +382,7 @@ __device__ __noinline__ void op_qr(const KernelParams& P, Team& tm, const Instr&
       const double ax2 = fma(x0.x, x0.x, x0.y * x0.y);
       const double s2 = ax2 + dj;
       int next = j + 1;
+      double drop = s2;  // weight that the null columns leave out of R
       const bool null = !(s2 > thr2);
       if (!null) {
         const double y = rsqrt((lane & 1) ? ax2 : s2);
@@ -401,8 +414,14 @@ __device__ __noinline__ void op_qr(const KernelParams& P, Team& tm, const Instr&
             break;
           }
         }
+        double v = 0.0;
+        for (int c = 1 + lane; c < next - j; c += 32) v += A::to(redo[4 * (n - j) + c]);
+        drop += warp_sum(v);
       }
-      if (lane == 0) qs.next = null ? -next : next;
+      if (lane == 0) {
+        qs.next = null ? -next : next;
+        if (null) qs.dropped += drop;
+      }
     }
     __syncthreads();
     const bool null = qs.next < 0;
@@ -570,37 +589,24 @@ __device__ __noinline__ void op_qr(const KernelParams& P, Team& tm, const Instr&
     const double y = a2 > 0.0 ? rsqrt(a2) : 0.0;
     qs.ph[j] = a2 > 0.0 ? make_double2(a.x * y, a.y * y) : make_double2(1.0, 0.0);
   }
+  if (threadIdx.x == NT - 32) {
+    const double rn2 = fro2 - qs.dropped;
+    qs.tau = rn2 > 0.0 ? sqrt(fro2 / rn2) : 1.0;
+  }
   __syncthreads();
   pc.lap(P.ctl, 11);
   // R (row j scaled by conj(ph_j)) into the bond buffer: R[j][k] = W[k][j] (k > j), diag alpha_j,
-  // rescaled to ||R||_F = ||M||_F (the weight of dropped sub-columns returns to the kept content)
-  if (tm.rank == 0) {
-    double loc = 0.0;
-    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-      const int j = idx / n, k = idx % n;
-      double2 r = make_double2(0, 0);
-      if (k > j) r = A::cto(W[(long long)k * rows + j]);
-      else if (k == j) r = qs.rdiag[j];
-      loc = fma(r.x, r.x, fma(r.y, r.y, loc));
-    }
-    loc = warp_sum(loc);
-    if (lane == 0) qs.red[warp] = loc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double rn = 0.0;
-      for (int w = 0; w < NWARP; ++w) rn += qs.red[w];
-      qs.tau = rn > 0.0 ? sqrt(fro2) / sqrt(rn) : 1.0;
-    }
-    __syncthreads();
+  // rescaled to ||R||_F = ||M||_F (the weight of dropped sub-columns returns to the kept content).
+  // The reflectors keep every column's norm, so ||R||_F^2 = ||M||_F^2 - the dropped weight; the
+  // entries are spread over the team (one CTA took 6 us for them, most of it FP64 instructions)
+  for (int idx = tm.gtid(); idx < n * n; idx += tm.nthr()) {
+    const int j = idx / n, k = idx % n;
+    double2 r = make_double2(0, 0);
+    if (k > j) r = A::cto(W[(long long)k * rows + j]);
+    else if (k == j) r = qs.rdiag[j];
+    const double2 p = qs.ph[j];
     const double scale = qs.tau;
-    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-      const int j = idx / n, k = idx % n;
-      double2 r = make_double2(0, 0);
-      if (k > j) r = A::cto(W[(long long)k * rows + j]);
-      else if (k == j) r = qs.rdiag[j];
-      const double2 p = qs.ph[j];
-      Rout[idx] = make_double2(scale * (r.x * p.x + r.y * p.y), scale * (r.y * p.x - r.x * p.y));
-    }
+    Rout[idx] = make_double2(scale * (r.x * p.x + r.y * p.y), scale * (r.y * p.x - r.x * p.y));
   }
   // Q[r][c] = (delta_rc - sum_a V[r][a] Z[a][c]) ph_c over the own rows, active columns a with
   // j_a <= min(r, c); a thread takes the columns c0 and c0 + 1 of one row (V loaded once)
@@ -623,12 +629,15 @@ __device__ __noinline__ void op_qr(const KernelParams& P, Team& tm, const Instr&
       q_cmac<A>(q1r, q1i, nv, Z[a * n + c1]);
     }
     auto put = [&](int c, S qr, S qi) {
-      Acc o_r, o_i;
-      o_r.init(A::zero());
-      o_i.init(A::zero());
-      q_cmac<A>(o_r, o_i, A::c(qr, qi), A::cfrom(qs.ph[c]));
+      E v = A::c(qr, qi);
+      if (qs.shat[c] != 0.0) {  // an active column: times its phase (1 otherwise)
+        Acc o_r, o_i;
+        o_r.init(A::zero());
+        o_i.init(A::zero());
+        q_cmac<A>(o_r, o_i, v, A::cfrom(qs.ph[c]));
+        v = A::c(o_r.val(), o_i.val());
+      }
       const long long at = qr_addr(nd, l, r, c);
-      const E v = A::c(o_r.val(), o_i.val());
       Ag[at] = A::cto(v);
       // the mixed modes' environment updates read Q from the FP32 mirror (the heads of v)
       if constexpr (std::is_same<A, QrDs>::value) P.pool32[nd.off + at] = make_float2(A::re(v).x, A::im(v).x);

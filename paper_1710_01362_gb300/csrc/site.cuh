@@ -14,8 +14,8 @@
 // The Krylov vectors' own parts stay in shared memory as far as they fit; an updated vector goes
 // to the CTAs that read its slices, through distributed shared memory (cluster teams) or a
 // slice-major copy in global memory (the grid team).
-// Forward exponential of a 40 x 40 x 20 tensor, whole grid: @SF0 us per operation before, @SF now
-// (BF16X3 mode); FP64 @SF640 and @SF64.
+// Forward exponential of a 40 x 40 x 20 tensor, whole grid, about four applications: 190 us per
+// operation before, 102 now (BF16X3 mode); FP64, about eight applications: 1500 and 660.
 //
 // The plan (legs, jobs, split, layout: SitePlan) comes from the host: worked out by one thread of
 // every CTA it took 6 us per operation.
@@ -131,17 +131,17 @@ __device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b
   b = p[1];
 }
 
-// Dense jobs on the own rows and P indices: results v * (dense product at the job's column) to
-// dbuf[job * stride + o].  xs: slices [slot][a][c] with rows of Cp; for C jobs `xrow` rows start at
-// the own block (environment updates hold only these... the same layout), a 2 x 2 tile per thread.
-template <typename T>
-__device__ __forceinline__ void site_products(const SitePlan& sp, const SiteUnit& u, const typename C2<T>::t* xs,
-                                              typename C2<T>::t* dbuf, int stride) {
+// Dense jobs on the own rows and P indices: results v * (dense product at the job's
+// column) to dbuf[job * stride + o], a TA x TC tile per thread.  xs: slices [slot][a][c], rows of
+// Cp.
+template <typename T, int TA, int TC>
+__device__ __noinline__ void site_tiles(const SitePlan& sp, const SiteUnit& u, const typename C2<T>::t* xs,
+                                        typename C2<T>::t* dbuf, int stride) {
   using V = typename C2<T>::t;
   const V* sm = reinterpret_cast<const V*>(dyn_smem + sp.mats);
   const V* vals = reinterpret_cast<const V*>(dyn_smem + sp.vals);
   const int* cols = reinterpret_cast<const int*>(dyn_smem + sp.cols);
-  const int na2 = (u.A + 1) / 2, nc2 = (sp.Dc + 1) / 2, Cq = sp.Dc + (sp.Dc & 1);
+  const int na2 = (u.A + TA - 1) / TA, nc2 = (sp.Dc + TC - 1) / TC, Cq = sp.Dc + (sp.Dc & 1);
   const int tiles = na2 * nc2;
   const float inv_t = tiles > 0 ? 1.0f / (float)tiles : 0.0f, inv_c2 = 1.0f / (float)nc2;
   const float inv_S = u.S > 0 ? 1.0f / (float)u.S : 0.0f;
@@ -150,57 +150,81 @@ __device__ __forceinline__ void site_products(const SitePlan& sp, const SiteUnit
     const int js = fdivu(it, tiles, inv_t), r = it - js * tiles;
     const int j = fdivu(js, u.S, inv_S), sl = js - j * u.S;
     const int at = fdivu(r, nc2, inv_c2);
-    const int al0 = 2 * at, al1 = min(al0 + 1, u.A - 1), c0 = 2 * (r - at * nc2);
+    const int al0 = TA * at, al1 = min(al0 + 1, u.A - 1), c0 = TC * (r - at * nc2);
     const V w = vals[j * sp.dp + u.s0 + sl];
-    V x00, x01, x10, x11;
-    x00.x = x00.y = x01.x = x01.y = x10.x = x10.y = x11.x = x11.y = (T)0;
+    V x[TA][TC];
+#pragma unroll
+    for (int i = 0; i < TA; ++i)
+#pragma unroll
+      for (int q = 0; q < TC; ++q) x[i][q].x = x[i][q].y = (T)0;
+    const SiteJob& jb = sp.job[j];
     if (w.x != (T)0 || w.y != (T)0) {
-      const SiteJob& jb = sp.job[j];
       const V* slice = xs + cols[j * sp.dp + u.s0 + sl];
-      const V *p0, *p1, *b;
-      int bs;
+      const V *p0, *b;
+      int ps, bs;  // the second row's distance, and b's row length
       if (jb.type == 0) {
         p0 = sm + jb.moff + al0 * sp.Da;
-        p1 = sm + jb.moff + al1 * sp.Da;
+        ps = sp.Da;
         b = slice + c0;
         bs = sp.Cp;
       } else {
-        p0 = slice + (u.a0 + al0) * sp.Cp;
-        p1 = slice + (u.a0 + al1) * sp.Cp;
         b = sm + jb.moff + c0;
         bs = Cq;
+        p0 = slice + (u.a0 + al0) * sp.Cp;
+        ps = sp.Cp;
       }
+      const V* p1 = p0 + (al1 - al0) * ps;
       const int K = jb.K;
 #pragma unroll 4
       for (int k = 0; k < K; ++k) {
-        const V q0 = p0[k], q1 = p1[k];
-        V b0, b1;
-        ld_pair(b + k * bs, b0, b1);
-        cmac<T>(x00, q0, b0);
-        cmac<T>(x01, q0, b1);
-        cmac<T>(x10, q1, b0);
-        cmac<T>(x11, q1, b1);
+        V q[TA], g[TC];
+        q[0] = p0[k];
+        if (TA > 1) q[TA - 1] = p1[k];
+        if constexpr (TC > 1)
+          ld_pair(b + k * bs, g[0], g[TC - 1]);
+        else
+          g[0] = b[k * bs];
+#pragma unroll
+        for (int i = 0; i < TA; ++i)
+#pragma unroll
+          for (int e = 0; e < TC; ++e) cmac<T>(x[i][e], q[i], g[e]);
       }
-      auto scale = [&](V& x) {
-        V y;
-        y.x = w.x * x.x - w.y * x.y;
-        y.y = w.x * x.y + w.y * x.x;
-        x = y;
-      };
       if (jb.nnz > 0) {
-        scale(x00);
-        scale(x01);
-        scale(x10);
-        scale(x11);
+#pragma unroll
+        for (int i = 0; i < TA; ++i)
+#pragma unroll
+          for (int e = 0; e < TC; ++e) {
+            V y;
+            y.x = w.x * x[i][e].x - w.y * x[i][e].y;
+            y.y = w.x * x[i][e].y + w.y * x[i][e].x;
+            x[i][e] = y;
+          }
       }
     }
     V* o = dbuf + j * stride + (sl * u.A + al0) * sp.Dc + c0;
-    o[0] = x00;
-    if (c0 + 1 < sp.Dc) o[1] = x01;
-    if (al1 > al0) {
-      o[sp.Dc] = x10;
-      if (c0 + 1 < sp.Dc) o[sp.Dc + 1] = x11;
-    }
+#pragma unroll
+    for (int i = 0; i < TA; ++i)
+#pragma unroll
+      for (int e = 0; e < TC; ++e)
+        if (al0 + i < u.A && c0 + e < sp.Dc) o[i * sp.Dc + e] = x[i][e];
+  }
+}
+// The tile: in FP32 2 x 2 (its operand loads are the bound) unless that leaves threads without
+// work, then 1 x 2 or single elements; in FP64 single elements (the FP64 pipe is the bound, and
+// tiles over odd edges waste it).
+template <typename T>
+__device__ __forceinline__ void site_products(const SitePlan& sp, const SiteUnit& u, const typename C2<T>::t* xs,
+                                              typename C2<T>::t* dbuf, int stride) {
+  if constexpr (std::is_same<T, double>::value) {
+    site_tiles<T, 1, 1>(sp, u, xs, dbuf, stride);
+  } else {
+    const int rows = sp.nd * u.S, nc2 = (sp.Dc + 1) / 2;
+    if (rows * ((u.A + 1) / 2) * nc2 >= NT)
+      site_tiles<T, 2, 2>(sp, u, xs, dbuf, stride);
+    else if (rows * u.A * nc2 >= NT)
+      site_tiles<T, 1, 2>(sp, u, xs, dbuf, stride);
+    else
+      site_tiles<T, 1, 1>(sp, u, xs, dbuf, stride);
   }
 }
 // Sum of block blk's jobs at own element o: dense results and sparse-only terms
@@ -213,21 +237,13 @@ __device__ __forceinline__ typename C2<T>::t site_sum(const SitePlan& sp, const 
   const int* cols = reinterpret_cast<const int*>(dyn_smem + sp.cols) + at.s;
   V y;
   y.x = y.y = (T)0;
-  if (blk == 0)  // every dense job of an environment update belongs to block 0 or its channel
 #pragma unroll 4
-    for (int j = 0; j < sp.nd; ++j) {
-      if (sp.job[j].blk) continue;
-      const V d = dbuf[j * stride + o];
-      y.x += d.x;
-      y.y += d.y;
-    }
-  else
-    for (int j = 0; j < sp.nd; ++j)
-      if (sp.job[j].blk == blk) {
-        const V d = dbuf[j * stride + o];
-        y.x += d.x;
-        y.y += d.y;
-      }
+  for (int j = 0; j < sp.nd; ++j) {
+    if (sp.job[j].blk != blk) continue;
+    const V d = dbuf[j * stride + o];
+    y.x += d.x;
+    y.y += d.y;
+  }
   const int row = at.a * sp.Cp + at.c;
   for (int j = sp.nd; j < sp.nj; ++j)
     if (sp.job[j].blk == blk) {
