@@ -7,6 +7,8 @@
 #include <cstddef>
 #include <cstring>
 #include <string>
+#include <functional>
+#include <queue>
 #include <unordered_map>
 #include <vector>
 
@@ -18,6 +20,11 @@ namespace ttns {
 cudaError_t launch_sweep(const KernelParams& P, int phase, int grid, int cluster, int cooperative,
                          cudaStream_t stream);
 cudaError_t max_grid_for(int cluster, long long smem_bytes, int* grid);
+namespace pair {
+cudaError_t launch_sweep(const KernelParams& P, int phase, int grid, int cluster, int cooperative,
+                         cudaStream_t stream);
+cudaError_t max_grid_for(int cluster, long long smem_bytes, int* grid);
+}  // namespace pair
 cudaError_t launch_density(const double2* pool, const NodeDesc& nd, int l, double* partials, int nblocks, double* out,
                            cudaStream_t st);
 cudaError_t launch_down(const double2* pool, const NodeDesc* d_nodes, const DownBatch& b, double* obs, double2* xbuf,
@@ -72,6 +79,8 @@ struct ttns_tree {
   Factor* d_chans = nullptr;
   Instr* d_prog = nullptr;
   TreeDesc* d_trees = nullptr;
+  int* d_order = nullptr;
+  bool pair = false;  // the kernel with two CTAs per SM
   SitePlan* d_sites = nullptr;
   std::vector<SitePlan> sites;
   Ctl* ctl = nullptr;
@@ -102,9 +111,13 @@ struct ttns_tree {
 // that drops the cluster shape of cooperative launches would give them) until the library has
 // switched to plain cluster launches; the kernel's launch check refuses each before any
 // barrier or distributed-shared-memory access.
+static cudaError_t launch_kernel(ttns_tree* t, const ttns::KernelParams& P, int phase, int cluster, int cooperative) {
+  const auto fn = t->pair ? ttns::pair::launch_sweep : ttns::launch_sweep;
+  return fn(P, phase, t->grid, cluster, cooperative, t->stream);
+}
 static cudaError_t launch_persistent(ttns_tree* t, const ttns::KernelParams& P, int phase) {
   const bool inject = (t->opt.launch_flags & 2) && !(t->opt.launch_flags & 1) && phase == 1;
-  return ttns::launch_sweep(P, phase, t->grid, inject ? 1 : t->cluster, !(t->opt.launch_flags & 1), t->stream);
+  return launch_kernel(t, P, phase, inject ? 1 : t->cluster, !(t->opt.launch_flags & 1));
 }
 
 static const char* kStatusNames[] = {"ok", "invalid", "oom", "cuda", "not converged", "timeout", "nonfinite", "io"};
@@ -298,6 +311,12 @@ static ttns_status check_tables(const Compiled& C, int mmax, long long kvec, lon
   return TTNS_OK;
 }
 
+// Limits of the kernel with two CTAs per SM.
+constexpr int kPairNode = 4096, kPairD = 40;
+constexpr double kPairSlow = 1.6;
+constexpr long long kPairSmem = 87 * 1024;
+static_assert(3LL * 2 * kPairD * kPairD * 8 <= kPairSmem, "QR reduction buffers exceed the shared memory");
+
 struct Sizes {
   int mmax;
   long long kvec, work_stride, per_cta;
@@ -348,12 +367,12 @@ static ttns_status wait_and_check(ttns_tree* t, bool phase0, const char* what) {
       KernelParams P0 = t->P;
       P0.dt = 0.0;
       P0.n_steps = 1;
-      CUDA_TRY(launch_sweep(P0, 0, t->grid, t->cluster, 0, t->stream));
+      CUDA_TRY(launch_kernel(t, P0, 0, t->cluster, 0));
     }
     for (const auto& pr : t->pending) {
       t->P.dt = pr.first;
       t->P.n_steps = pr.second;
-      CUDA_TRY(launch_sweep(t->P, 1, t->grid, t->cluster, 0, t->stream));
+      CUDA_TRY(launch_kernel(t, t->P, 1, t->cluster, 0));
     }
     CUDA_TRY(cudaStreamSynchronize(t->stream));
     CUDA_TRY(cudaMemcpy(&h, t->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
@@ -367,7 +386,8 @@ static ttns_status wait_and_check(ttns_tree* t, bool phase0, const char* what) {
 // every row-sparse factor on the remaining leg P (environment updates: A is the instruction's leg
 // and carries no dense factor).  Returns false where the form or the shared memory does not fit;
 // the operation then takes the general path.
-static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize, long long smem, SitePlan* out) {
+static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize, long long smem, SitePlan* out,
+                      bool* no_room) {
   const NodeDesc& nd = C.nodes[I.node];
   const bool env = I.op == OP_ENV;
   if ((I.op != OP_FWD && !env) || nd.nl < 2 || nd.nl > 3) return false;
@@ -494,7 +514,10 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
   off += sp.nd * own * (long long)vsize;
   if (env) off += (1LL + I.nchan) * sp.sb * sp.Ab * sp.Cp * (long long)vsize;
   off = up(off);
-  if (off > smem) return false;
+  if (off > smem) {
+    *no_room = true;
+    return false;
+  }
   sp.rest = (int)off;
   *out = sp;
   return true;
@@ -502,10 +525,12 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
 
 // Site plans of the whole program: one per distinct operation (the same node, leg and team recur
 // in a step), equal plans of different nodes shared.
-static void build_site_plans(ttns_tree* t, int grid, long long smem) {
+// Returns false if the shared memory was too small for one of them.
+static bool build_site_plans(ttns_tree* t, int grid, long long smem) {
   Compiled& C = t->C;
   t->sites.clear();
   const size_t vsize = t->opt.precision == TTNS_FP64 ? sizeof(double2) : sizeof(float2);
+  bool no_room = false;
   constexpr int kNone = -2;
   std::vector<int> by_op(C.lists.size() * 4, kNone);
   std::unordered_multimap<unsigned long long, int> by_plan;
@@ -524,7 +549,7 @@ static void build_site_plans(ttns_tree* t, int grid, long long smem) {
       continue;
     }
     SitePlan sp;
-    if (site_plan(C, I, I.team == TEAM_GRID ? grid : t->cluster, vsize, smem, &sp)) {
+    if (site_plan(C, I, I.team == TEAM_GRID ? grid : t->cluster, vsize, smem, &sp, &no_room)) {
       unsigned long long h = 1469598103934665603ULL;
       words(sp, [&](const char* b, size_t n) {
         for (size_t k = 0; k + 8 <= n; k += 8) {
@@ -545,6 +570,24 @@ static void build_site_plans(ttns_tree* t, int grid, long long smem) {
     }
     known = I.site;
   }
+  return !no_room;
+}
+
+// Completion time of a set of trees (costs in decreasing order) on n clusters, each taking the
+// next tree when it is done with one.
+static double makespan(const std::vector<double>& cost, int n) {
+  std::priority_queue<double, std::vector<double>, std::greater<double>> busy;
+  double end = 0.0;
+  for (double c : cost) {
+    double at = 0.0;
+    if ((int)busy.size() >= n) {
+      at = busy.top();
+      busy.pop();
+    }
+    busy.push(at + c);
+    end = std::max(end, at + c);
+  }
+  return end;
 }
 
 static ttns_status device_init(ttns_tree* t) {
@@ -558,11 +601,36 @@ static ttns_status device_init(ttns_tree* t) {
   t->cluster = o.cluster_ctas > 0 ? o.cluster_ctas : 16;
   if (t->cluster > 16) return fail(TTNS_E_INVALID, "cluster_ctas must be <= 16");
   int maxgrid = 0;
-  const long long smem_bytes = 201 * 1024;  // with the kernel's static shared memory, all of an SM's 227 KB
+  long long smem_bytes = 201 * 1024;  // with the kernel's static shared memory, all of an SM's 227 KB
   // the QR keeps three reduction buffers of 2 n^2 doubles (n <= TTNS_MAX_D) in it
   static_assert(3LL * 2 * TTNS_MAX_D * TTNS_MAX_D * 8 <= 200 * 1024, "QR reduction buffers exceed the shared memory");
   CUDA_TRY(max_grid_for(t->cluster, smem_bytes, &maxgrid));
   if (maxgrid < t->cluster) return fail(TTNS_E_CUDA, "no co-resident cluster of the requested size");
+  // trees by decreasing program length, which is what their time follows
+  std::vector<int> order(C.trees.size());
+  for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int a, int b) { return C.trees[a].prog_count > C.trees[b].prog_count; });
+  // Two CTAs per SM where it shortens the whole set: beside another one a cluster takes 1.16
+  // (four-CTA teams) to 1.6 times as long (one-CTA teams), so the set has to gain more than
+  // that from twice the clusters.  Not for tensors from the size at which the tensor-core
+  // products start, nor where a plan or the QR's buffers need more than half the shared memory:
+  // FP64 chains of D 12-24 on one CTA took 2906 ms instead of 1960 when their plans did not fit.
+  // Measured, one CTA per SM against two: 256 chains on four CTAs 218 and 136 ms, on eight 439 and
+  // 214; 304 ER trees of D 8 91 and 73 ms (TF32X3), 184 and 133 (FP64); 64 chains on four CTAs
+  // (36 clusters fit) 99 and 102.
+  if (t->batched && o.grid_ctas <= 0 && C.max_node < kPairNode && C.max_D <= kPairD) {
+    std::vector<double> cost;
+    for (int k : order) cost.push_back(C.trees[k].prog_count);
+    int pairs = 0;
+    CUDA_TRY(pair::max_grid_for(t->cluster, kPairSmem, &pairs));
+    if (pairs >= t->cluster && kPairSlow * makespan(cost, pairs / t->cluster) < makespan(cost, maxgrid / t->cluster) &&
+        build_site_plans(t, pairs, kPairSmem)) {
+      t->pair = true;
+      smem_bytes = kPairSmem;
+      maxgrid = pairs;
+    }
+  }
   int grid = o.grid_ctas > 0 ? o.grid_ctas : maxgrid;
   grid = std::min(grid, maxgrid);
   grid = (grid / t->cluster) * t->cluster;
@@ -583,10 +651,11 @@ static ttns_status device_init(ttns_tree* t) {
   if ((s = upload(t, &t->d_terms, C.terms)) != TTNS_OK) return s;
   if ((s = upload(t, &t->d_lists, C.lists)) != TTNS_OK) return s;
   if ((s = upload(t, &t->d_chans, C.chans)) != TTNS_OK) return s;
-  build_site_plans(t, grid, smem_bytes);
+  if (!t->pair) build_site_plans(t, grid, smem_bytes);
   if ((s = upload(t, &t->d_sites, t->sites)) != TTNS_OK) return s;
   if ((s = upload(t, &t->d_prog, C.prog)) != TTNS_OK) return s;
   if ((s = upload(t, &t->d_trees, C.trees)) != TTNS_OK) return s;
+  if ((s = upload(t, &t->d_order, order)) != TTNS_OK) return s;
   if ((s = dalloc(t, &t->ctl, 1)) != TTNS_OK) return s;
   CUDA_TRY(cudaMemsetAsync(t->ctl, 0, sizeof(Ctl), t->stream));
   if ((s = dalloc(t, &t->work, (size_t)n_workers * work_stride)) != TTNS_OK) return s;
@@ -622,6 +691,7 @@ static ttns_status device_init(ttns_tree* t) {
   P.prog = t->d_prog;
   P.trees = t->d_trees;
   P.sites = t->d_sites;
+  P.order = t->d_order;
   P.n_trees = (int)C.trees.size();
   P.batched = t->batched ? 1 : 0;
   P.ctl = t->ctl;
@@ -986,7 +1056,7 @@ static ttns_status run_phase(ttns_tree* t, int phase, const char* what) {
   KernelParams Pp = t->P;
   Pp.dt = 0.0;
   Pp.n_steps = 1;
-  CUDA_TRY(launch_sweep(Pp, phase, t->grid, t->cluster, !(t->opt.launch_flags & 1), t->stream));
+  CUDA_TRY(launch_kernel(t, Pp, phase, t->cluster, !(t->opt.launch_flags & 1)));
   CUDA_TRY(cudaStreamSynchronize(t->stream));
   Ctl h;
   CUDA_TRY(cudaMemcpy(&h, t->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
@@ -995,7 +1065,7 @@ static ttns_status run_phase(ttns_tree* t, int phase, const char* what) {
     ++t->launch_fallbacks;
     h.status = h.err_where = h.err_node = 0;
     CUDA_TRY(cudaMemcpy(t->ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice));
-    CUDA_TRY(launch_sweep(Pp, phase, t->grid, t->cluster, 0, t->stream));
+    CUDA_TRY(launch_kernel(t, Pp, phase, t->cluster, 0));
     CUDA_TRY(cudaStreamSynchronize(t->stream));
     CUDA_TRY(cudaMemcpy(&h, t->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
   }

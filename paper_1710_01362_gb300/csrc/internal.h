@@ -143,6 +143,7 @@ struct KernelParams {
   const Instr* prog;
   const TreeDesc* trees;
   const SitePlan* sites;
+  const int* order;        // batched: trees by decreasing program length
   int n_trees;
   int batched;             // 1: each cluster runs whole trees; 0: one tree, mixed teams
   Ctl* ctl;

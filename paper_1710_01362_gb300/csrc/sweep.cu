@@ -13,6 +13,10 @@
 //   * reductions are deterministic: per-CTA partials, then a fixed-order sum
 //     that every CTA computes identically (no floating-point atomics);
 //   * every spin-wait is bounded and reports TTNS_E_TIMEOUT instead of hanging.
+//
+// Two instances of the kernel are compiled from this file: one CTA per SM with all of its
+// registers and shared memory, and (SWEEP_PAIR, from sweep_pair.cu) two CTAs per SM for sets of
+// many small trees.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -26,7 +30,16 @@
 
 namespace cg = cooperative_groups;
 
+#ifdef SWEEP_PAIR
+#define SWEEP_CTAS 2
+#else
+#define SWEEP_CTAS 1
+#endif
+
 namespace ttns {
+#ifdef SWEEP_PAIR
+namespace pair {
+#endif
 
 #define NT 256
 #define NWARP (NT / 32)
@@ -1273,7 +1286,7 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
   // tensor-core apply (split precision) for nodes whose terms have one dense factor each; its
   // operand tiles take the dynamic shared memory, so nothing staged there is used
   bool use_tc = false;
-  if (s_tc.on && (P.precision == 1 || P.precision == 2) && N >= 4096) {
+  if (SWEEP_CTAS == 1 && s_tc.on && (P.precision == 1 || P.precision == 2) && N >= 4096) {
     if (threadIdx.x == 0) {
       tc_plan(nd, os, L, P.precision == 2 ? tc::Split<tc::KIND_BF16X3>::kstep / 2 : tc::Split<tc::KIND_TF32X3>::kstep / 2,
               s_tcp);
@@ -1724,8 +1737,19 @@ __device__ void run(const KernelParams& P, int phase) {
   ct.csize = cs;
   double2* cwork = P.work + (long long)cluster_id * P.work_stride;
   if (P.batched) {
-    for (int tree = cluster_id; tree < P.n_trees; tree += n_clusters) {
-      const TreeDesc& td = P.trees[tree];
+    // A cluster takes the next tree when it is done with one, the long programs first.  Every
+    // launch draws n_trees + n_clusters tickets (one too many per cluster), so the counter
+    // needs no reset; batched launches have no grid barrier that would use it.
+    __shared__ int s_ticket;
+    for (;;) {
+      __syncthreads();
+      if (threadIdx.x == 0 && crank == 0)
+        s_ticket = (int)(atomicAdd(&P.ctl->bar_count, 1ull) % (unsigned long long)(P.n_trees + n_clusters));
+      if (cs > 1) cg::this_cluster().sync(); else __syncthreads();
+      const int ticket = cs > 1 ? *cg::this_cluster().map_shared_rank(&s_ticket, 0) : s_ticket;
+      if (cs > 1) cg::this_cluster().sync();  // read before rank 0 draws again or leaves
+      if (ticket >= P.n_trees) break;
+      const TreeDesc& td = P.trees[P.order[ticket]];
       const int first = phase == 0 ? td.init_first : (phase == 2 ? td.obs_first : (phase == 3 ? td.grow_first : td.prog_first));
       const int count = phase == 0 ? td.init_count : (phase == 2 ? td.obs_count : (phase == 3 ? td.grow_count : td.prog_count));
       const int nst = phase == 1 ? P.n_steps : 1;
@@ -1783,7 +1807,13 @@ __device__ __forceinline__ unsigned sreg_dynamic_smem_size() {
   return r;
 }
 
-__global__ void __launch_bounds__(NT, 1) k_sweep(KernelParams P, int phase) {
+// The two-CTA instance: what bounds batches of small trees is latency (FP64 chains, cluster
+// barriers, scalar steps on one warp), and a second tree on the SM fills the waits.  It has half
+// the registers and shared memory and no tensor memory (its trees are below the size at which
+// the tensor-core products start).  One step of 256 chains of 10 to 40 sites on four-CTA teams
+// (TF32X3): 327 ms before (trees in order, one per cluster at a time), 218 with the longest first
+// on whichever cluster is free, 136 with two CTAs per SM.
+__global__ void __launch_bounds__(NT, SWEEP_CTAS) k_sweep(KernelParams P, int phase) {
   // Launch self-check before any barrier or distributed-shared-memory access: the
   // interpreter addresses cluster peers by rank and stages operands up to smem_bytes, so a
   // launch with another cluster shape or less dynamic shared memory returns an error
@@ -1795,7 +1825,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep(KernelParams P, int phase) {
     return;
   }
   // tensor memory for the split-precision contractions (one 128-column accumulator per CTA)
-  const bool tc_on = P.precision == 1 || P.precision == 2;
+  const bool tc_on = SWEEP_CTAS == 1 && (P.precision == 1 || P.precision == 2);
   if (threadIdx.x == 0) s_tc.on = 0;
   if (tc_on) {
     if ((threadIdx.x >> 5) == 0) tc::tmem_alloc(&s_tc.tmem, kTcTmemCols);
@@ -1821,6 +1851,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweep(KernelParams P, int phase) {
   }
 }
 
+#ifndef SWEEP_PAIR
 // ------------------------------------------------------------------ observables
 // Density of a root leg: partials of rho[b][b2] = sum_rows A[row, b] conj(A[row, b2]) along leg l,
 // rows split over the blocks
@@ -2006,10 +2037,12 @@ cudaError_t launch_mirror32(const double2* pool, float2* pool32, long long n, cu
   return cudaGetLastError();
 }
 
+#endif
+
 // ------------------------------------------------------------------ host launch helpers
 static bool g_tables_set = false;
 
-cudaError_t upload_constants() {
+static cudaError_t upload_constants() {
   if (g_tables_set) return cudaSuccess;
   double inv[256], invf[128];
   inv[0] = 0.0;
@@ -2071,6 +2104,7 @@ cudaError_t max_grid_for(int cluster, long long smem_bytes, int* grid) {
   return cudaSuccess;
 }
 
+#ifndef SWEEP_PAIR
 cudaError_t launch_density(const double2* pool, const NodeDesc& nd, int l, double* partials, int nblocks, double* out,
                            cudaStream_t st) {
   k_density_partial<<<nblocks, NT, 0, st>>>(pool + nd.off, nd, l, partials);
@@ -2087,4 +2121,8 @@ cudaError_t launch_energy(const KernelParams& P, int node, int terms, int n2, do
   return cudaGetLastError();
 }
 
+#endif
+#ifdef SWEEP_PAIR
+}  // namespace pair
+#endif
 }  // namespace ttns
