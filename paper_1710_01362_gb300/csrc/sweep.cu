@@ -669,8 +669,17 @@ __device__ void team_reduce_vec(Team& tm, const double* mine, double* out, int n
 // with h = (nl - 1) / 2.  A term is computed in the pass whose tile holds all its legs, from
 // the tile of the input vector staged in shared memory (every element of a tile is read by
 // D of its neighbours along a leg: this replaces strided L2 reads).  Pass A writes its sum,
-// pass B adds its terms to it.  Two-stage terms, or a term with legs in neither tile, keep
-// the element-wise apply.
+// pass B adds its terms to it.  A term with legs in neither tile keeps the element-wise apply.
+//
+// In FP32 a dense factor is a product over the fibres of its leg in the tile, a block of rows and
+// fibres per thread (tile_product), and a two-factor term is that product followed by the other
+// factor on its result: element by element the operand loads are the bound (two shared-memory
+// or L2 words per multiply-add).  Root of a star of four chains (20^4 x 5, two of the couplings
+// with three entries a row, which kept it from being tiled), whole grid, TF32X3 mode: 5760 us per
+// exponential before, 3410 now.  In FP64 the FP64 pipe is the bound in either form (18.9 ms
+// element by element, 20.5 by products), so there, and where three tiles (input, sum, product)
+// do not fit in shared memory, a tile's terms are taken element by element, without two-stage
+// terms.
 struct TiledApply {
   NodeDesc ta, tb;                  // the tile tensors of the two passes
   int h;
@@ -686,7 +695,7 @@ __shared__ TiledApply s_tp;
 
 __device__ void tiled_plan(const NodeDesc& nd, const OpStage& os, const TermList& L, TiledApply& tp) {
   const int nl = nd.nl, h = (nl - 1) / 2;
-  tp.ok = nl >= 3 && h >= 1 && L.n2 == 0 && L.count <= 64;
+  tp.ok = nl >= 3 && h >= 1 && L.count <= 64;
   if (!tp.ok) return;
   tp.h = h;
   NodeDesc& a = tp.ta;
@@ -735,14 +744,103 @@ __device__ void tiled_plan(const NodeDesc& nd, const OpStage& os, const TermList
       if (allB) tp.inB |= 1ull << t;
       else tp.ok = 0;
     }
+    if (tt.nf == 2 && tt.f[0].nnz > 0 && tt.f[1].nnz > 0) tp.ok = 0;
   }
 }
 
-// One pass over this CTA's tiles; emit(global index, sum of the pass's terms at it).
+// out (+)= M x along one leg of a tile of TT elements: dimension D, stride st; TA rows times TC
+// fibres per thread.
+template <typename T, int TA, int TC>
+__device__ __forceinline__ void tile_rows(const typename C2<T>::t* M, int D, int st, float inv_st, int TT,
+                                          const typename C2<T>::t* x, typename C2<T>::t* out, bool add) {
+  using V = typename C2<T>::t;
+  const int nc = TT / D, ncg = (nc + TC - 1) / TC, nrg = (D + TA - 1) / TA;
+  const float inv_g = 1.0f / (float)ncg;
+  for (int it = threadIdx.x; it < nrg * ncg; it += NT) {
+    const int rg = fdivu(it, ncg, inv_g), c0 = it - rg * ncg, i0 = rg * TA;
+    int base[TC];
+    const V* row[TA];
+    V acc[TA][TC];
+#pragma unroll
+    for (int q = 0; q < TC; ++q) {
+      const int c = min(c0 + q * ncg, nc - 1), hi = fdivu(c, st, inv_st);
+      base[q] = hi * D * st + c - hi * st;
+    }
+#pragma unroll
+    for (int i = 0; i < TA; ++i) {
+      row[i] = M + min(i0 + i, D - 1) * D;
+#pragma unroll
+      for (int q = 0; q < TC; ++q) acc[i][q].x = acc[i][q].y = (T)0;
+    }
+#pragma unroll 4
+    for (int k = 0; k < D; ++k) {
+      V m[TA], v[TC];
+#pragma unroll
+      for (int i = 0; i < TA; ++i) m[i] = row[i][k];
+#pragma unroll
+      for (int q = 0; q < TC; ++q) v[q] = x[base[q] + k * st];
+#pragma unroll
+      for (int i = 0; i < TA; ++i)
+#pragma unroll
+        for (int q = 0; q < TC; ++q) cmac<T>(acc[i][q], m[i], v[q]);
+    }
+#pragma unroll
+    for (int i = 0; i < TA; ++i)
+#pragma unroll
+      for (int q = 0; q < TC; ++q)
+        if (i0 + i < D && c0 + q * ncg < nc) {
+          V* o = out + base[q] + (i0 + i) * st;
+          V r = acc[i][q];
+          if (add) {
+            r.x += o->x;
+            r.y += o->y;
+          }
+          *o = r;
+        }
+  }
+}
+// The block: 4 x 2 (6 loads for 8 multiply-adds) unless that leaves threads without work.
+template <typename T>
+__device__ __noinline__ void tile_product(const KernelParams& P, const NodeDesc& td, const OpStage& os, const Factor& f,
+                                          int leg, const typename C2<T>::t* x, typename C2<T>::t* out, bool add) {
+  using V = typename C2<T>::t;
+  const int D = td.dims[leg], st = td.strides[leg], TT = td.size;
+  const int slot = fslot(os, f, D);
+  const V* M = slot >= 0 ? reinterpret_cast<const V*>(dyn_smem) + slot : ops<T>(P) + f.mat;
+  const float inv_st = td.inv_strides[leg];
+  if (TT >= 8 * NT || (TT >= 6 * NT && D % 4 == 0))
+    tile_rows<T, 4, 2>(M, D, st, inv_st, TT, x, out, add);
+  else if (TT >= 4 * NT)
+    tile_rows<T, 2, 2>(M, D, st, inv_st, TT, x, out, add);
+  else
+    tile_rows<T, 1, 1>(M, D, st, inv_st, TT, x, out, add);
+}
+
+// Shared memory of the tiled apply, or nullptr: three tiles (fibres), or the input tile alone
+// for lists without two-stage terms.  The same on every CTA.  any: with fewer tiles than CTAs too.
+template <typename T>
+__device__ typename C2<T>::t* tiled_begin(const KernelParams& P, const Team& tm, const NodeDesc& nd, const OpStage& os,
+                                          const TermList& L, bool any, bool& tiled, bool& fibres) {
+  TiledApply& tp = s_tp;
+  if (threadIdx.x == 0) tiled_plan(nd, os, L, tp);
+  __syncthreads();
+  tiled = fibres = false;
+  if (!tp.ok || (!any && (std::is_same<T, double>::value || min(tp.nta, tp.ntb) < tm.size))) return nullptr;
+  const int TT = tp.ta.size > tp.tb.size ? tp.ta.size : tp.tb.size;
+  typename C2<T>::t* xt = nullptr;
+  if constexpr (!std::is_same<T, double>::value) xt = vec_smem<T>(P, os, 3LL * TT);
+  fibres = xt != nullptr;
+  if (!fibres && L.n2 == 0) xt = vec_smem<T>(P, os, TT);
+  tiled = xt != nullptr;
+  return xt;
+}
+
+// One pass over this CTA's tiles; emit(global index, sum of the pass's terms at it).  xt: the
+// input tile, with `fibres` followed by the tile's sum and a factor's result.
 template <typename T, typename F>
 __device__ void tiled_pass(const KernelParams& P, Team& tm, const TiledApply& tp, const OpStage& os,
-                           const TermList& L, const typename C2<T>::t* xin, typename C2<T>::t* xt, int pass,
-                           F&& emit) {
+                           const TermList& L, const typename C2<T>::t* xin, typename C2<T>::t* xt, bool fibres,
+                           int pass, F&& emit) {
   using V = typename C2<T>::t;
   const NodeDesc& td = pass ? tp.tb : tp.ta;
   const int* lmap = pass ? tp.lmapB : tp.lmapA;
@@ -774,8 +872,58 @@ __device__ void tiled_pass(const KernelParams& P, Team& tm, const TiledApply& tp
       }
     }
     __syncthreads();  // the previous tile's reads are done
-    for (int e = threadIdx.x; e < TT; e += NT) xt[e] = xin[gidx(base, e)];
+    for (int e = threadIdx.x; e < TT; e += NT) {
+      if constexpr (sizeof(V) == 16)
+        cp_async16(xt + e, xin + gidx(base, e));
+      else
+        cp_async8(xt + e, xin + gidx(base, e));
+    }
+    cp_async_wait_all();
     __syncthreads();
+    if constexpr (!std::is_same<T, double>::value) if (fibres) {
+      V* y = xt + TT;
+      V* z = y + TT;
+      for (int e = threadIdx.x; e < TT; e += NT) {  // terms of one sparse factor
+        V acc;
+        acc.x = acc.y = (T)0;
+        for (int t = 0; t < L.count; ++t) {
+          if ((int)((tp.inB >> t) & 1ull) != pass || os.terms[t].nf != 1 || os.terms[t].f[0].nnz == 0) continue;
+          Factor f = os.terms[t].f[0];
+          f.leg = lmap[f.leg];
+          const V a = factor_dot<T>(P, td, f, os, xt, e);
+          acc.x += a.x;
+          acc.y += a.y;
+        }
+        y[e] = acc;
+      }
+      __syncthreads();
+      for (int t = 0; t < L.count; ++t) {
+        const Term& tt = os.terms[t];
+        if ((int)((tp.inB >> t) & 1ull) != pass) continue;
+        if (tt.nf == 1) {
+          if (tt.f[0].nnz > 0) continue;
+          tile_product<T>(P, td, os, tt.f[0], lmap[tt.f[0].leg], xt, y, true);
+          __syncthreads();
+          continue;
+        }
+        const int d = tt.f[0].nnz == 0 ? 0 : 1;  // a dense factor first (tiled_plan: there is one)
+        tile_product<T>(P, td, os, tt.f[d], lmap[tt.f[d].leg], xt, z, false);
+        __syncthreads();
+        Factor f = tt.f[1 - d];
+        f.leg = lmap[f.leg];
+        if (f.nnz == 0)
+          tile_product<T>(P, td, os, f, f.leg, z, y, true);
+        else
+          for (int e = threadIdx.x; e < TT; e += NT) {
+            const V a = factor_dot<T>(P, td, f, os, z, e);
+            y[e].x += a.x;
+            y[e].y += a.y;
+          }
+        __syncthreads();
+      }
+      for (int e = threadIdx.x; e < TT; e += NT) emit(gidx(base, e), y[e]);
+      continue;
+    }
     for (int e = threadIdx.x; e < TT; e += NT) {
       V acc;
       acc.x = acc.y = (T)0;
@@ -1310,15 +1458,8 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
   // tiled apply for a grid-team node that does not fit in shared memory
   TiledApply& tp = s_tp;
   V* xt = nullptr;
-  bool tiled = false;
-  if (tm.kind == TEAM_GRID && xs == nullptr && !use_tc) {
-    if (threadIdx.x == 0) tiled_plan(nd, os, L, tp);
-    __syncthreads();
-    if (tp.ok) {
-      xt = vec_smem<T>(P, os, tp.ta.size > tp.tb.size ? tp.ta.size : tp.tb.size);
-      tiled = xt != nullptr;  // the same on every CTA
-    }
-  }
+  bool tiled = false, fibres = false;
+  if (tm.kind == TEAM_GRID && xs == nullptr && !use_tc) xt = tiled_begin<T>(P, tm, nd, os, L, L.n2 == 0, tiled, fibres);
   pc.lap(P.ctl, 0);
   // exp(-i s H): s = time / hbar with the op's sign.  If the Krylov space of dimension
   // mmax does not reach the tolerance for the remaining time, the largest s / 2^k that
@@ -1358,7 +1499,7 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
       }
       // operand of this application: shared memory, the FP32 shadow, or K_j itself (FP64)
       const V* xin = xs ? xs : (shadow ? xf : reinterpret_cast<const V*>(Kj));
-      if (L.n2 > 0) {
+      if (L.n2 > 0 && !tiled) {
         apply_stage1<T>(P, tm, nd, xin, L, tmp, kv, os);
         team_sync(tm);
       }
@@ -1386,10 +1527,10 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
         for (long long idx = tm.gtid(); idx < N; idx += tm.nthr())
           recur(idx, tc_sum_at<T>(P, nd, os, s_tcp, xin, ybuf, kv, idx));
       } else if (tiled) {
-        V* y = tmp;  // pass A sums (no two-stage terms, so the temporaries are free)
-        tiled_pass<T>(P, tm, tp, os, L, xin, xt, 0, [&](long long g, V acc) { y[g] = acc; });
+        V* y = tmp;  // pass A sums (the temporaries of two-stage terms are not used here)
+        tiled_pass<T>(P, tm, tp, os, L, xin, xt, fibres, 0, [&](long long g, V acc) { y[g] = acc; });
         team_sync(tm);
-        tiled_pass<T>(P, tm, tp, os, L, xin, xt, 1, [&](long long g, V acc) {
+        tiled_pass<T>(P, tm, tp, os, L, xin, xt, fibres, 1, [&](long long g, V acc) {
           V a = y[g];
           a.x += acc.x;
           a.y += acc.y;
@@ -1496,6 +1637,120 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
 // contracted over every leg of Q except the leg toward v.  This form takes the tensors that are
 // not sites (ER nodes, roots of several chains, OBB sites): results of all rows in global memory,
 // every output value summed over all rows by one CTA.
+// Projection of the grid team: out[b][a][a'] = sum_rows conj(Q[row, a]) Y_b[row, a'].  Every CTA
+// sums over its own rows, in blocks of kProjRows staged in shared memory with a 2 x 2 tile of
+// outputs per thread, in runs of one block in the compute type and between blocks in FP64 or
+// double-single; the CTAs' partials are added in order.  With outputs split over the CTAs instead
+// (below) every CTA reads all rows, a word per multiply-add from L2: 417 us at 40000 rows, D 20, in
+// FP32 and 780 in FP64; 70 and 434 now.  From a block of rows per CTA on; with fewer the partials
+// and their sum cost as much as the products.
+constexpr int kProjRows = 64;
+template <typename T>
+__device__ __noinline__ bool project_rows(const KernelParams& P, Team& tm, const Instr& I, const NodeDesc& nd,
+                                          const typename C2<T>::t* xq, const typename C2<T>::t* Y) {
+  using V = typename C2<T>::t;
+  using A = typename EnvArith<T>::A;
+  using E = typename A::E;
+  const int l = I.leg, D = I.D, nch = I.nchan, nb = 1 + nch, lst = nd.strides[l];
+  const int rows = nd.size / D, chunk = (rows + tm.size - 1) / tm.size;
+  const long long kv = P.kvec;
+  constexpr int RP = kProjRows + 1;  // odd: lanes on different columns read different banks
+  if (tm.kind != TEAM_GRID || rows < kProjRows * tm.size || 2LL * D * RP * (long long)sizeof(V) > P.smem_bytes) return false;
+  V* Qs = reinterpret_cast<V*>(dyn_smem);
+  V* Ys = Qs + D * RP;
+  const int rb = min(rows, tm.rank * chunk), re = min(rows, rb + chunk);
+  const int D2 = D * D, nval = nb * D2, h = (D + 1) / 2;
+  const float inv_h = 1.0f / (float)h, inv_D = nd.inv_dims[l], inv_l = nd.inv_strides[l];
+  E* buf = reinterpret_cast<E*>(team_partials(tm));
+  E* mine = buf + (long long)tm.rank * nval;
+  auto load = [&](V* dst, const V* src, int r0, int nr) {  // dst[a][r]
+    const float inv_n = 1.0f / (float)nr;
+    for (int it = threadIdx.x; it < D * nr; it += NT) {
+      int a, r;
+      if (lst == 1) {
+        r = fdivu(it, D, inv_D);
+        a = it - r * D;
+      } else {
+        a = fdivu(it, nr, inv_n);
+        r = it - a * nr;
+      }
+      const int p = fdivu(r0 + r, lst, inv_l);
+      const V* g = src + (long long)p * D * lst + (r0 + r - p * lst) + (long long)a * lst;
+      if constexpr (sizeof(V) == 16)
+        cp_async16(dst + a * RP + r, g);
+      else
+        cp_async8(dst + a * RP + r, g);
+    }
+  };
+  auto skip = [&](int b) { return b > 0 && ((I.adj >> (b - 1)) & 1u); };  // adjoint of the channel before
+  for (int r0 = rb; r0 < re || r0 == rb; r0 += kProjRows) {
+    const int nr = max(0, min(kProjRows, re - r0));
+    for (int b = 0; b < nb; ++b) {
+      if (skip(b)) continue;
+      __syncthreads();
+      if (nr > 0) {
+        if (b == 0) load(Qs, xq, r0, nr);
+        load(Ys, Y + b * kv, r0, nr);
+      }
+      cp_async_wait_all();
+      __syncthreads();
+      for (int it = threadIdx.x; it < h * h; it += NT) {
+        const int ta = fdivu(it, h, inv_h);
+        const int a0 = 2 * ta, a1 = min(a0 + 1, D - 1), p0 = 2 * (it - ta * h), p1 = min(p0 + 1, D - 1);
+        const V *q0 = Qs + a0 * RP, *q1 = Qs + a1 * RP, *y0 = Ys + p0 * RP, *y1 = Ys + p1 * RP;
+        V s[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[q].x = s[q].y = (T)0;
+        auto cj = [](V& e, V q, V y) {  // e += conj(q) y
+          e.x = fma(q.x, y.x, fma(q.y, y.y, e.x));
+          e.y = fma(q.x, y.y, fma(-q.y, y.x, e.y));
+        };
+#pragma unroll 4
+        for (int r = 0; r < nr; ++r) {
+          const V u0 = q0[r], u1 = q1[r], w0 = y0[r], w1 = y1[r];
+          cj(s[0], u0, w0);
+          cj(s[1], u0, w1);
+          cj(s[2], u1, w0);
+          cj(s[3], u1, w1);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int a = a0 + (q >> 1), p = p0 + (q & 1);
+          if (a >= D || p >= D) continue;
+          E& e = mine[b * D2 + a * D + p];
+          E o = r0 == rb ? A::c(A::zero(), A::zero()) : e;
+          if constexpr (std::is_same<T, double>::value)
+            o = A::c(A::add(A::re(o), s[q].x), A::add(A::im(o), s[q].y));
+          else
+            o = A::c(A::add(A::re(o), make_float2(s[q].x, 0.f)), A::add(A::im(o), make_float2(s[q].y, 0.f)));
+          e = o;
+        }
+      }
+    }
+  }
+  team_sync(tm);
+  double2* out = P.pool + I.env_out;
+  auto emit = [&](int k, E v) {
+    out[k] = A::cto(v);
+    if constexpr (!std::is_same<T, double>::value) P.pool32[I.env_out + k] = make_float2(A::re(v).x, A::im(v).x);
+  };
+  for (int k = tm.gtid(); k < nval; k += tm.nthr()) {
+    const int b = k / D2, r = k - b * D2, a = r / D, p = r - a * D;
+    if (skip(b)) continue;
+    typename A::S sr = A::zero(), si = A::zero();
+#pragma unroll 8
+    for (int q = 0; q < tm.size; ++q) {
+      const E v = buf[(long long)q * nval + k];
+      sr = A::add(sr, A::re(v));
+      si = A::add(si, A::im(v));
+    }
+    emit(k, A::c(sr, si));
+    if (b > 0 && b < nch && ((I.adj >> b) & 1u)) emit((b + 1) * D2 + p * D + a, A::c(sr, A::neg(si)));
+  }
+  tm.parity ^= 1;
+  return true;
+}
+
 template <typename T>
 __device__ __noinline__ void op_env(const KernelParams& P, Team& tm, const Instr& I, double2* work) {
   const NodeDesc nd = P.nodes[I.node];
@@ -1529,23 +1784,36 @@ __device__ __noinline__ void op_env(const KernelParams& P, Team& tm, const Instr
     xq = reinterpret_cast<const V*>(Q);
   }
   pc.lap(P.ctl, 16);
-  if (L.n2 > 0) {
+  bool tiled = false, fibres = false;
+  V* xt = nullptr;
+  if (tm.kind == TEAM_GRID && xs == nullptr) xt = tiled_begin<T>(P, tm, nd, os, L, false, tiled, fibres);
+  if (tiled) {
+    tiled_pass<T>(P, tm, s_tp, os, L, xq, xt, fibres, 0, [&](long long g, V acc) { Y[g] = acc; });
+    team_sync(tm);
+    tiled_pass<T>(P, tm, s_tp, os, L, xq, xt, fibres, 1, [&](long long g, V acc) {
+      V a = Y[g];
+      a.x += acc.x;
+      a.y += acc.y;
+      Y[g] = a;
+    });
+  } else if (L.n2 > 0) {
     apply_stage1<T>(P, tm, nd, xq, L, tmp, kv, os);
     team_sync(tm);
   }
   for (long long idx = tm.gtid(); idx < N; idx += tm.nthr()) {
-    Y[idx] = apply_stage2_at<T>(P, nd, xq, L, tmp, kv, idx, os);
+    if (!tiled) Y[idx] = apply_stage2_at<T>(P, nd, xq, L, tmp, kv, idx, os);
     for (int b = 0; b < I.nchan; ++b) Y[(long long)(1 + b) * kv + idx] = factor_dot<T>(P, nd, os.chans[b], os, xq, idx);
   }
   team_sync(tm);
   pc.lap(P.ctl, 17);
+  const bool projected = xs == nullptr && project_rows<T>(P, tm, I, nd, xq, Y);  // (stages in xs's place)
   // projection: out[b][a][a'] = sum_rows conj(Q[row, a]) Y_b[row, a'].  Each CTA owns a
   // contiguous block of the output values and sums them over all rows: the rows of an output
   // are split into `parts` ranges over the CTA's threads (partial sums in the compute type in
   // runs of 64 rows, then FP64), and one thread per output adds its parts in a fixed order and
   // writes the value; no partial sums cross CTAs.
   const long long rows = N / D;
-  const int nval = nb * D * D;
+  const int nval = projected ? 0 : nb * D * D;
   const long long lst = nd.strides[l];
   const int opc = (nval + tm.size - 1) / tm.size;
   const int ob = min(nval, tm.rank * opc), oe = min(nval, ob + opc);
