@@ -799,7 +799,8 @@ __device__ __forceinline__ void tile_rows(const typename C2<T>::t* M, int D, int
         }
   }
 }
-// The block: 4 x 2 (6 loads for 8 multiply-adds) unless that leaves threads without work.
+// The block with the fewest operand loads per thread (rounds x (rows + fibres)): 4 x 2 at D 20 and
+// 5 D^2 elements, 2 x 2 at D 14 (one round instead of four of single elements).
 template <typename T>
 __device__ __noinline__ void tile_product(const KernelParams& P, const NodeDesc& td, const OpStage& os, const Factor& f,
                                           int leg, const typename C2<T>::t* x, typename C2<T>::t* out, bool add) {
@@ -808,9 +809,12 @@ __device__ __noinline__ void tile_product(const KernelParams& P, const NodeDesc&
   const int slot = fslot(os, f, D);
   const V* M = slot >= 0 ? reinterpret_cast<const V*>(dyn_smem) + slot : ops<T>(P) + f.mat;
   const float inv_st = td.inv_strides[leg];
-  if (TT >= 8 * NT || (TT >= 6 * NT && D % 4 == 0))
+  const int nc = TT / D, nc2 = (nc + 1) / 2;
+  auto loads = [](int items, int per) { return (items + NT - 1) / NT * per; };
+  const int l1 = loads(TT, 2), l2 = loads((D + 1) / 2 * nc2, 4), l4 = loads((D + 3) / 4 * nc2, 6);
+  if (l4 < l2 && l4 < l1)
     tile_rows<T, 4, 2>(M, D, st, inv_st, TT, x, out, add);
-  else if (TT >= 4 * NT)
+  else if (l2 < l1)
     tile_rows<T, 2, 2>(M, D, st, inv_st, TT, x, out, add);
   else
     tile_rows<T, 1, 1>(M, D, st, inv_st, TT, x, out, add);
@@ -1431,10 +1435,21 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
   OpStage& os = s_os;
   stage_op<T>(P, I, L, nullptr, 0, os);
   using V = typename C2<T>::t;
+  constexpr bool kShadow = !std::is_same<T, double>::value;
   // tensor-core apply (split precision) for nodes whose terms have one dense factor each; its
   // operand tiles take the dynamic shared memory, so nothing staged there is used
-  bool use_tc = false;
-  if (SWEEP_CTAS == 1 && s_tc.on && (P.precision == 1 || P.precision == 2) && N >= 4096) {
+  // (a large root's tiles first: 2980 us per exponential at 20^4 x 5, the tensor cores 4210 in
+  // TF32X3 and 3550 in BF16X3, where splitting the operands is the bound; 980 us at 14^4 x 5, 980
+  // and 1030 there.  With fewer tiles than
+  // CTAs the tensor cores are ahead: 400 us at 20^3 x 5, by tiles 580)
+  V* xt = nullptr;
+  bool tiled = false, fibres = false, use_tc = false;
+  if constexpr (kShadow)
+    if (tm.kind == TEAM_GRID && vec_smem<T>(P, os, N) == nullptr) {
+      xt = tiled_begin<T>(P, tm, nd, os, L, false, tiled, fibres);
+      tiled = fibres;
+    }
+  if (SWEEP_CTAS == 1 && !fibres && s_tc.on && (P.precision == 1 || P.precision == 2) && N >= 4096) {
     if (threadIdx.x == 0) {
       tc_plan(nd, os, L, P.precision == 2 ? tc::Split<tc::KIND_BF16X3>::kstep / 2 : tc::Split<tc::KIND_TF32X3>::kstep / 2,
               s_tcp);
@@ -1447,19 +1462,16 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
     use_tc = s_tcp.ok != 0;
   }
   V* ybuf = reinterpret_cast<V*>(work + (long long)(P.mmax + P.n_tmp + 2) * kv);  // group results (TC)
-  V* xs = use_tc ? nullptr : vec_smem<T>(P, os, N);  // input vector in shared memory when it fits
+  V* xs = use_tc || fibres ? nullptr : vec_smem<T>(P, os, N);  // input vector in shared memory when it fits
   // otherwise, in mixed precision, a compute-type copy of the input vector in the workspace,
   // written by the pass that produces the vector (FP64 Krylov basis, FP32 operand)
   // (kept in the mixed modes whether or not the vector is staged: staging then copies it
   // instead of converting the FP64 vector on every CTA)
-  constexpr bool kShadow = !std::is_same<T, double>::value;
   V* xf = reinterpret_cast<V*>(work + (long long)(P.mmax + P.n_tmp) * kv);
   const bool shadow = kShadow;
   // tiled apply for a grid-team node that does not fit in shared memory
   TiledApply& tp = s_tp;
-  V* xt = nullptr;
-  bool tiled = false, fibres = false;
-  if (tm.kind == TEAM_GRID && xs == nullptr && !use_tc) xt = tiled_begin<T>(P, tm, nd, os, L, L.n2 == 0, tiled, fibres);
+  if (tm.kind == TEAM_GRID && xs == nullptr && !use_tc && !fibres) xt = tiled_begin<T>(P, tm, nd, os, L, L.n2 == 0, tiled, fibres);
   pc.lap(P.ctl, 0);
   // exp(-i s H): s = time / hbar with the op's sign.  If the Krylov space of dimension
   // mmax does not reach the tolerance for the remaining time, the largest s / 2^k that
