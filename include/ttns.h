@@ -59,7 +59,8 @@ typedef enum {
  * 2^-44 relative per operation, FP32's exponent range) in the other modes.
  *   TTNS_FP64    every contraction in FP64;
  *   TTNS_TF32X3  split-precision tensor cores: the H_eff applications of tensors of at least 4096
- *                elements whose terms have one dense factor each are complex GEMMs on tcgen05 with
+ *                elements whose terms have one dense factor each, other than chain sites and
+ *                roots that have a tile for every CTA, are complex GEMMs on tcgen05 with
  *                3xTF32 operands (hi*hi + hi*lo + lo*hi) and FP32 accumulation in tensor memory;
  *                every other contraction in FP32 on the SIMT cores;
  *   TTNS_BF16X3  the same with a 3-way BF16 split and the 6 products of order <= 2^-16;

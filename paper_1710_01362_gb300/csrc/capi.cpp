@@ -8,6 +8,7 @@
 #include <cstring>
 #include <string>
 #include <functional>
+#include <new>
 #include <queue>
 #include <unordered_map>
 #include <vector>
@@ -397,9 +398,10 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
     int blk;
     const Factor *d, *s;
   };
-  std::vector<Pair> prs;
-  prs.reserve(L.count + 16);
+  Pair prs[kSiteJobs];
+  int np = 0;
   auto add = [&](int blk, const Factor* a, const Factor* b) {
+    if (np == kSiteJobs) return false;
     Pair pr{blk, nullptr, nullptr};
     for (const Factor* f : {a, b}) {
       if (!f) continue;
@@ -407,7 +409,7 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
       if (slot) return false;
       slot = f;
     }
-    prs.push_back(pr);
+    prs[np++] = pr;
     return true;
   };
   for (int k = 0; k < L.count; ++k) {
@@ -419,14 +421,16 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
       if (!add(1 + b, &C.chans[I.chan_first + b], nullptr)) return false;
   unsigned dense = 0, sparse = 0;
   int nj = 0;
-  for (const Pair& pr : prs) {
+  for (int k = 0; k < np; ++k) {
+    const Pair& pr = prs[k];
     if (pr.d) dense |= 1u << pr.d->leg;
     if (pr.s) sparse |= 1u << pr.s->leg;
     nj += pr.s ? pr.s->nnz : 1;
   }
   if (nj > kSiteJobs || (sparse & (sparse - 1))) return false;
-  SitePlan sp;
-  std::memset(&sp, 0, sizeof(sp));
+  SitePlan& sp = *out;  // (its parts in use: a large set of trees has tens of thousands of plans)
+  std::memset(&sp, 0, offsetof(SitePlan, job));
+  std::memset(sp.job, 0, sizeof(SiteJob) * nj);
   sp.P = nd.nl - 1;
   for (int q = 0; q < nd.nl; ++q)
     if ((sparse >> q) & 1u) sp.P = q;
@@ -437,7 +441,8 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
   for (int q = 0; q < nd.nl; ++q)
     if (q != sp.P && q != sp.A) sp.C = q;
   for (int pass = 0; pass < 2; ++pass) {
-    for (const Pair& pr : prs) {
+    for (int k = 0; k < np; ++k) {
+      const Pair& pr = prs[k];
       if ((pr.d != nullptr) != (pass == 0)) continue;
       for (int q = 0; q < (pr.s ? pr.s->nnz : 1); ++q) {
         SiteJob& j = sp.job[sp.nj++];
@@ -519,7 +524,6 @@ static bool site_plan(const Compiled& C, const Instr& I, int team, size_t vsize,
     return false;
   }
   sp.rest = (int)off;
-  *out = sp;
   return true;
 }
 
@@ -539,6 +543,11 @@ static bool build_site_plans(ttns_tree* t, int grid, long long smem) {
     fn(b, offsetof(SitePlan, need) + sizeof(sp.need[0]) * sp.ns);
     fn(b + offsetof(SitePlan, job), sizeof(SiteJob) * sp.nj);
   };
+  auto same = [](const SitePlan& a, const SitePlan& b) {
+    return std::memcmp(&a, &b, offsetof(SitePlan, job)) == 0 && std::memcmp(a.job, b.job, sizeof(SiteJob) * a.nj) == 0;
+  };
+  SitePlan sp;
+  std::memset(&sp, 0, sizeof(sp));
   for (Instr& I : C.prog) {
     I.site = -1;
     if (I.op != OP_FWD && I.op != OP_ENV) continue;
@@ -548,7 +557,6 @@ static bool build_site_plans(ttns_tree* t, int grid, long long smem) {
       I.site = known;
       continue;
     }
-    SitePlan sp;
     if (site_plan(C, I, I.team == TEAM_GRID ? grid : t->cluster, vsize, smem, &sp, &no_room)) {
       unsigned long long h = 1469598103934665603ULL;
       words(sp, [&](const char* b, size_t n) {
@@ -561,7 +569,7 @@ static bool build_site_plans(ttns_tree* t, int grid, long long smem) {
       });
       const auto range = by_plan.equal_range(h);
       for (auto it = range.first; it != range.second && I.site < 0; ++it)
-        if (std::memcmp(&t->sites[it->second], &sp, sizeof(sp)) == 0) I.site = it->second;
+        if (same(t->sites[it->second], sp)) I.site = it->second;
       if (I.site < 0) {
         I.site = (int)t->sites.size();
         t->sites.push_back(sp);
@@ -590,7 +598,7 @@ static double makespan(const std::vector<double>& cost, int n) {
   return end;
 }
 
-static ttns_status device_init(ttns_tree* t) {
+static ttns_status device_init(ttns_tree* t) try {
   Compiled& C = t->C;
   const ttns_options& o = t->opt;
   Sizes z;
@@ -723,6 +731,8 @@ static ttns_status device_init(ttns_tree* t) {
   // initial environment pass
   CUDA_TRY(launch_persistent(t, P, 0));
   return wait_and_check(t, true, "device status after the initial pass: ");
+} catch (const std::bad_alloc&) {  // host tables
+  return fail(TTNS_E_OOM, "host allocation failed");
 }
 
 static ttns_status check_options(const ttns_options& o) {

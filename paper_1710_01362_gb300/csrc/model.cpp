@@ -684,6 +684,14 @@ struct TreeCompiler {
     };
     return a.va == b.va && a.vb == b.vb && adj(a.opa, b.opa) && adj(a.opb, b.opb);
   }
+  // whether coupling k is the adjoint of coupling j; neighbours (the usual case) are compared once
+  std::vector<signed char> adj_prev;
+  bool adjoint_of(int j, int k) {
+    if (j != k - 1) return adjoint_pair(t.coups[j], t.coups[k]);
+    if (adj_prev.empty()) adj_prev.assign(t.coups.size(), -1);
+    if (adj_prev[k] < 0) adj_prev[k] = adjoint_pair(t.coups[j], t.coups[k]) ? 1 : 0;
+    return adj_prev[k] > 0;
+  }
   void emit_env(int u, int v) {
     auto key = std::make_pair(u, v);
     auto it = envh_list.find(key);
@@ -714,7 +722,7 @@ struct TreeCompiler {
     I.nchan = env_chan[key].second;
     // the two halves of a hopping term follow each other: the second block is the first's adjoint
     for (int c = 1; c < I.nchan && c < 32; ++c)
-      if (!((I.adj >> (c - 1)) & 1u) && adjoint_pair(t.coups[E.chans[c - 1]], t.coups[E.chans[c]])) I.adj |= 1u << c;
+      if (!((I.adj >> (c - 1)) & 1u) && adjoint_of(E.chans[c - 1], E.chans[c])) I.adj |= 1u << c;
     I.env_out = E.off;
     I.D = E.D;
     I.flops = list_flops(li, C.nodes[I.node]) + 8.0 * C.nodes[I.node].size * E.D * (1 + E.chans.size());
