@@ -96,14 +96,6 @@ struct DsAcc {
   __device__ __forceinline__ float2 val() const { return ds_quick(s, c); }
 };
 
-// complex accumulators: (ar, ai) += a b
-__device__ __forceinline__ void ds_cmac(DsAcc& ar, DsAcc& ai, float4 a, float4 b) {
-  ar.mac(ds_re(a), ds_re(b));
-  ar.mac(ds_neg(ds_im(a)), ds_im(b));
-  ai.mac(ds_re(a), ds_im(b));
-  ai.mac(ds_im(a), ds_re(b));
-}
-
 __device__ __forceinline__ float2 shfl_xor_ds(float2 v, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }

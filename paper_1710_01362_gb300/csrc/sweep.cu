@@ -180,14 +180,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   return __shfl_sync(0xffffffffu, v, 0);
 }
 
-template <int NV>
-__device__ __forceinline__ void warp_sum_n(double* v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-}
-
 // Sum of V values (a power of two <= 16) over a warp with V - 1 + 5 - log2(V) additions per
 // lane instead of 5 V: the first log2(V) butterfly levels exchange half of the remaining
 // values, the rest are plain.  Lane L returns the total of value warp_reduce_vid<V>(L); the
@@ -1439,9 +1431,9 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
   // tensor-core apply (split precision) for nodes whose terms have one dense factor each; its
   // operand tiles take the dynamic shared memory, so nothing staged there is used
   // (a large root's tiles first: 2980 us per exponential at 20^4 x 5, the tensor cores 4210 in
-  // TF32X3 and 3550 in BF16X3, where splitting the operands is the bound; 980 us at 14^4 x 5, 980
-  // and 1030 there.  With fewer tiles than
-  // CTAs the tensor cores are ahead: 400 us at 20^3 x 5, by tiles 580)
+  // TF32X3 and 3550 in BF16X3, where splitting the operands is the bound; at 14^4 x 5 980 us, there
+  // 980 and 1030.  With fewer tiles than CTAs the tensor cores are ahead: 400 us at 20^3 x 5, by
+  // tiles 580)
   V* xt = nullptr;
   bool tiled = false, fibres = false, use_tc = false;
   if constexpr (kShadow)
