@@ -131,9 +131,13 @@ __device__ __noinline__ void texp_warp(const double* a, const double* b, int m, 
   const int lane = threadIdx.x & 31;
   const bool on = lane < m;
   ChebSetup cs = cheb_setup(a, b, m, fabsf((float)s));
-  const double c = (double)cs.c;
+  const double c = m > 1 ? (double)cs.c : a[0];  // one component: the phase alone
   double vre = lane == 0 ? 1.0 : 0.0, vim = 0.0;
-  if (cs.R > 0.f && cs.z < 1e4f && cs.z > 0.f) {  // (non-finite input: the caller reports it)
+  if (m > 1 && cs.R > 0.f && cs.z >= 1e4f) {
+    // hundreds of sub-steps on one warp, for a time that no Krylov space of this size covers:
+    // NaN, which the caller reports (a vector left at e_0 would pass its convergence check)
+    vre = vim = __longlong_as_double(0x7ff8000000000000LL);
+  } else if (m > 1 && cs.R > 0.f && cs.z > 0.f) {  // (a NaN in the input reaches the result through c)
     // sub-steps of |z| <= 28: the order stays below 64
     const int nsub = (int)ceilf(cs.z * (1.0f / 28.0f));
     const double R = (double)cs.R;
