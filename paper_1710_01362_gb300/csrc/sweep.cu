@@ -687,8 +687,9 @@ __shared__ TiledApply s_tp;
 
 __device__ void tiled_plan(const NodeDesc& nd, const OpStage& os, const TermList& L, TiledApply& tp) {
   const int nl = nd.nl, h = (nl - 1) / 2;
-  tp.ok = nl >= 3 && h >= 1 && L.count <= 64;
-  if (!tp.ok) return;
+  tp.ok = 0;
+  if (nl < 3 || h < 1 || L.count > 64) return;
+  bool ok = true;
   tp.h = h;
   NodeDesc& a = tp.ta;
   a.nl = nl - h;
@@ -734,10 +735,11 @@ __device__ void tiled_plan(const NodeDesc& nd, const OpStage& os, const TermList
     }
     if (!allA) {
       if (allB) tp.inB |= 1ull << t;
-      else tp.ok = 0;
+      else ok = false;
     }
-    if (tt.nf == 2 && tt.f[0].nnz > 0 && tt.f[1].nnz > 0) tp.ok = 0;
+    if (tt.nf == 2 && tt.f[0].nnz > 0 && tt.f[1].nnz > 0) ok = false;
   }
+  tp.ok = ok;
 }
 
 // out (+)= M x along one leg of a tile of TT elements: dimension D, stride st; TA rows times TC
@@ -814,10 +816,13 @@ __device__ __noinline__ void tile_product(const KernelParams& P, const NodeDesc&
 
 // Shared memory of the tiled apply, or nullptr: three tiles (fibres), or the input tile alone
 // for lists without two-stage terms.  The same on every CTA.  any: with fewer tiles than CTAs too.
+// The plan is shared: the barrier before it waits for the readers of an earlier one (an
+// exponential may ask twice), and a caller that changes `os` afterwards needs one of its own.
 template <typename T>
 __device__ typename C2<T>::t* tiled_begin(const KernelParams& P, const Team& tm, const NodeDesc& nd, const OpStage& os,
                                           const TermList& L, bool any, bool& tiled, bool& fibres) {
   TiledApply& tp = s_tp;
+  __syncthreads();
   if (threadIdx.x == 0) tiled_plan(nd, os, L, tp);
   __syncthreads();
   tiled = fibres = false;
@@ -1440,6 +1445,7 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
     if (tm.kind == TEAM_GRID && vec_smem<T>(P, os, N) == nullptr) {
       xt = tiled_begin<T>(P, tm, nd, os, L, false, tiled, fibres);
       tiled = fibres;
+      __syncthreads();  // every thread has placed its tiles by os.end, which the plan below clears
     }
   if (SWEEP_CTAS == 1 && !fibres && s_tc.on && (P.precision == 1 || P.precision == 2) && N >= 4096) {
     if (threadIdx.x == 0) {
