@@ -2116,7 +2116,9 @@ __global__ void __launch_bounds__(NT, SWEEP_CTAS) k_sweep(KernelParams P, int ph
     __syncthreads();
     tc::fence_after();
   }
-  __syncthreads();
+  // the first operation writes to its peers' shared memory: every CTA of the cluster has to have
+  // started (and cleared its tensor-core record) by then
+  if (ncta > 1) cg::this_cluster().sync(); else __syncthreads();
   if (P.precision == 0)
     run<double>(P, phase);
   else
