@@ -1584,6 +1584,51 @@ ttns_status read_header(FILE* f, std::vector<TreeInput>* ins, int* record, int* 
   return TTNS_OK;
 }
 
+// The operators of a state file replace the built ones, and a file of another problem of the same
+// shape may have its entries in other columns.  Takes over the row-sparse tables that the
+// operations use, and where one differs makes the site plans again: they hold which slices a CTA
+// reads.  A column outside its leg gives TTNS_E_IO and leaves the tree as it was.
+ttns_status adopt_tables(ttns_tree* t, const std::vector<double2>& pool) {
+  Compiled& C = t->C;
+  std::vector<std::pair<long long, long long>> changed;  // offset, length
+  std::vector<char> seen(C.lists.size(), 0);
+  bool ok = true;
+  auto look = [&](const Factor& f, const NodeDesc& nd) {
+    if (f.nnz == 0) return;
+    const long long D = nd.dims[f.leg], n = D * f.nnz;
+    for (long long e = 0; e < n; ++e) {
+      const double c = pool[f.sp + n + e].x;
+      ok = ok && c >= 0.0 && c < (double)D;
+    }
+    if (std::memcmp(&pool[f.sp], &C.pool_init[f.sp], sizeof(double2) * 2 * n) != 0) changed.emplace_back(f.sp, 2 * n);
+  };
+  for (const Instr& I : C.prog) {
+    if ((I.op != OP_FWD && I.op != OP_BOND && I.op != OP_ENV) || seen[I.terms]) continue;
+    seen[I.terms] = 1;  // (a list belongs to one node and operator)
+    const NodeDesc& nd = C.nodes[I.node];
+    const TermList& L = C.lists[I.terms];
+    for (int k = 0; k < L.count; ++k)
+      for (int j = 0; j < C.terms[L.first + k].nf; ++j) look(C.terms[L.first + k].f[j], nd);
+    if (I.op == OP_ENV)
+      for (int b = 0; b < I.nchan; ++b) look(C.chans[I.chan_first + b], nd);
+  }
+  if (!ok) return fail(TTNS_E_IO, "checkpoint: a sparse operator's column is out of range");
+  if (changed.empty()) return TTNS_OK;
+  for (const auto& c : changed) std::copy_n(pool.begin() + c.first, c.second, C.pool_init.begin() + c.first);
+  build_site_plans(t, t->grid, t->P.smem_bytes);
+  t->allocs.erase(std::find(t->allocs.begin(), t->allocs.end(), (void*)t->d_sites));
+  cudaFree(t->d_sites);
+  ttns_status s = upload(t, &t->d_sites, t->sites);
+  if (s != TTNS_OK) {  // the general forms, which need no plan
+    t->d_sites = nullptr;
+    for (Instr& I : C.prog) I.site = -1;
+  }
+  t->P.sites = t->d_sites;
+  CUDA_TRY(cudaMemcpyAsync(t->d_prog, C.prog.data(), C.prog.size() * sizeof(Instr), cudaMemcpyHostToDevice, t->stream));
+  CUDA_TRY(cudaStreamSynchronize(t->stream));
+  return TTNS_OK;
+}
+
 // Reads the state section into an existing tree set of the same shape.
 ttns_status read_state(ttns_tree* t, FILE* f) {
   long long hdr[4];
@@ -1601,6 +1646,7 @@ ttns_status read_state(ttns_tree* t, FILE* f) {
             std::fread(mh.data(), sizeof(int), mh.size(), f) == mh.size() &&
             std::fread(tc.data(), sizeof(int), tc.size(), f) == tc.size() && std::fread(&h, sizeof(Ctl), 1, f) == 1;
   if (!ok) return fail(TTNS_E_IO, "checkpoint truncated");
+  if (const ttns_status s = adopt_tables(t, pool); s != TTNS_OK) return s;
   // the tensors are not validated here: a non-finite entry is reported by the next step
   // (TTNS_E_NONFINITE from the Krylov norm)
   h.bar_count = 0;
