@@ -157,7 +157,8 @@ __global__ void __launch_bounds__(kNT, 2) k_mlp_gemm(GemmArgs g) {
   __shared__ uint32_t tbase_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int split = gridDim.z;  // = cluster size along z
-  const int m0 = blockIdx.x * kTM, n0 = blockIdx.y * NP;
+  const unsigned row_tiles = (unsigned)((g.M - 1) / kTM) + 1u;  // (tiles on x: y ends at 65535)
+  const int m0 = (int)(blockIdx.x % row_tiles) * kTM, n0 = (int)(blockIdx.x / row_tiles) * NP;
   // this CTA's part of K: whole groups of K steps
   const int steps = (g.K + KS - 1) / KS;
   const int per = ((steps + split - 1) / split + kGroup - 1) / kGroup * kGroup;
@@ -347,7 +348,9 @@ cudaError_t launch_tile(GemmArgs g, int split, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_mlp_gemm<KIND, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((g.M + kTM - 1) / kTM, (g.N + NP - 1) / NP, split);
+  const long long tiles = ((g.M + (long long)kTM - 1) / kTM) * ((g.N + (long long)NP - 1) / NP);
+  if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  cfg.gridDim = dim3((unsigned)tiles, 1, split);
   cfg.blockDim = dim3(kNT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
