@@ -145,23 +145,26 @@ __device__ __noinline__ void texp_warp(const double* a, const double* b, int m, 
     cheb_order(cs, (float)z);
     const int K = cs.K;
     // Bessel functions J_n(z), n < 64 (lane n and n - 32), by backward recurrence from an order
-    // beyond K, normalised by J_0 + 2 sum J_2k = 1 (Miller's algorithm)
+    // beyond K, normalised by J_0 + 2 sum J_2k = 1 (Miller's algorithm).  The factor 2 n / z is
+    // formed anew at every order: stepped down by 2 / z its error reaches N roundings of the first
+    // factor at the small orders, which carry the norm (error of the exponential at z = 3: 6.6e-15
+    // against 7e-16).  J_0 is what the others leave of 1, to half a rounding for small z.
     double J0 = 0.0, J1 = 0.0;
     if (z > 1e-9) {
       const int N = ((K + 9) / 2) * 2;
       const double h = 2.0 / z;
-      double f = 1e-30, f1 = 0.0, sum = 0.0, cn = (double)N * h;
-      for (int n = N; n >= 0; --n) {
+      double f = 1e-30, f1 = 0.0, even = 0.0, dn = (double)N;
+      for (int n = N; n > 0; --n) {
         if (n == lane) J0 = f;
         if (n == lane + 32) J1 = f;
-        if ((n & 1) == 0) sum += f;
-        const double fm = fma(cn, f, -f1);
-        cn -= h;
+        if ((n & 1) == 0) even += f;
+        const double fm = fma(dn * h, f, -f1);
+        dn -= 1.0;
         f1 = f;
         f = fm;
       }
-      const double inv = 1.0 / (2.0 * sum - f1);  // f1: order 0
-      J0 *= inv;
+      const double inv = 1.0 / fma(2.0, even, f);  // f: order 0
+      J0 = lane == 0 ? fma(-2.0 * inv, even, 1.0) : J0 * inv;
       J1 *= inv;
     } else {  // the first two terms of each power series
       J0 = lane == 0 ? 1.0 : (lane == 1 ? 0.5 * z : (lane == 2 ? 0.125 * z * z : 0.0));
