@@ -52,3 +52,26 @@ def test_a_long_step_is_covered_by_substeps(name, dt):
     g.step(dt, 1)
     assert np.abs(g.rho() - o.rho_el()).max() < 1e-7
     g.close()
+
+
+# narrow and wide spectra for the Krylov dimension, halved times, tolerances near and far from FP32's
+# resolution: the spaces end where the oracle's FP64 estimate ends them (its check starts at the
+# first step; the library's at a leading-order bound, never later in these runs)
+@pytest.mark.parametrize("name,dt,mmax,tol", [("chain", 0.5, 30, 1e-12), ("chain", 20.0, 30, 1e-12), ("chain", 20.0, 6, 1e-9),
+                                              ("star", 5.0, 12, 1e-12), ("star", 1.0, 30, 1e-6), ("chain", 0.5, 30, 1e-14)])
+def test_krylov_spaces_end_where_the_oracle_ends_them(name, dt, mmax, tol):
+    p = TREES[name][0]()
+    o = TTNS(p, tol=tol, mmax=mmax)
+    o.step(dt)
+    g = ttns.Tree(p, precision=ttns.TTNS_FP64, krylov_mmax=mmax, krylov_tol=tol)
+    g.step(dt, 1)
+    if o.stats.get("not_converged"):  # 64 spaces do not cover the step: the library reports it
+        with pytest.raises(ttns.TTNSError) as e:
+            g.sync()
+        assert e.value.code == 4
+        g.close()
+        return
+    g.sync()
+    n = g.counters()["krylov_iters"]
+    g.close()
+    assert abs(n - o.stats["krylov_iters"]) <= 0.02 * o.stats["krylov_iters"], (n, o.stats)
