@@ -218,18 +218,20 @@ __device__ __noinline__ void texp_warp(const double* a, const double* b, int m, 
 // Convergence of step m: beta_m |e_m^T exp(-i s T_m) e_0| <= tol, decided as the FP64 expansion
 // decides it.  That takes 4 us and more on one warp, so an FP32 estimate comes first and answers
 // where it is certain.  Component m has no contribution from orders below m - 1, and the series of
-// an order n loses about z^2 / (2 n) / ln 10 digits to cancellation: with z^2 <= 12 m the estimate
-// is good to 1.3e-4 however small the component is (6500 random and Krylov matrices of m = 2 to 30
-// against FP64; beyond z^2 = 30 m it can be off by any factor).  Within 1 % of the tolerance, with
-// wider spectra and for tolerances near FP32's range the FP64 expansion decides: one step more or
-// less changes what is left below the tolerance, and the QR's null decisions can amplify that.
+// an order n loses about z^2 / (2 n) / ln 10 digits to cancellation.  For components of 1e-15 and
+// more the estimate was off by at most 6e-4 up to z^2 = 12 m and 6e-3 up to 20 m (15000 random and
+// Krylov matrices of m = 2 to 32 against FP64; beyond 30 m it can be off by any factor).  Within 1 %
+// or 5 % of the tolerance, with wider spectra and for smaller tolerances the FP64 expansion decides:
+// one step more or less changes what is left below the tolerance, and the QR's null decisions can
+// amplify that.  (With 12 m as the limit, 256 chains of up to 40 sites took 4.8 % longer.)
 __device__ __noinline__ bool krylov_small(const KrylovShared& ks, int m, double s, double tol, double* ure,
                                           double* uim, bool* nonfinite) {
   const int lane = threadIdx.x & 31;
   const double bn = ks.beta[m];
   ChebSetup cs = cheb_setup(ks.alpha, ks.beta, m, fabsf((float)s));
   *nonfinite = false;
-  if (cs.z * cs.z <= 12.f * (float)m && tol >= 1e-15 * bn) {
+  const float width = cs.z * cs.z / (float)m;
+  if (width <= 20.f && tol >= 1e-15 * bn) {
     cheb_order(cs, cs.z);
     const int K = min(64, cs.K + 4);
     const float y = -0.25f * cs.z * cs.z;
@@ -259,8 +261,9 @@ __device__ __noinline__ bool krylov_small(const KrylovShared& ks, int m, double 
     float um = 2.f * sqrtf(E * E + O * O) * 9.094947017729282e-13f;
     um = __shfl_sync(0xffffffffu, um, m - 1);
     const double err = bn * (double)um;
-    if (err <= 0.99 * tol) return true;
-    if (err >= 1.01 * tol) return !(bn > 0.0);
+    const double margin = width <= 12.f ? 0.01 : 0.05;
+    if (err <= (1.0 - margin) * tol) return true;
+    if (err >= (1.0 + margin) * tol) return false;
   }
   texp_warp(ks.alpha, ks.beta, m, s, ure, uim);
   const double r = ure[m - 1], i = uim[m - 1];
