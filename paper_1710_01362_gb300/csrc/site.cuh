@@ -175,8 +175,15 @@ __device__ __noinline__ void site_tiles(const SitePlan& sp, const SiteUnit& u, c
       }
       const V* p1 = p0 + (al1 - al0) * ps;
       const int K = jb.K;
-#pragma unroll 4
-      for (int k = 0; k < K; ++k) {
+      constexpr int U = std::is_same<T, double>::value ? 1 : 4;
+      V acc[TA][TC][U];
+#pragma unroll
+      for (int i = 0; i < TA; ++i)
+#pragma unroll
+        for (int e = 0; e < TC; ++e)
+#pragma unroll
+          for (int u4 = 0; u4 < U; ++u4) acc[i][e][u4].x = acc[i][e][u4].y = (T)0;
+      auto step = [&](int k, int u4) {
         V q[TA], g[TC];
         q[0] = p0[k];
         if (TA > 1) q[TA - 1] = p1[k];
@@ -187,8 +194,18 @@ __device__ __noinline__ void site_tiles(const SitePlan& sp, const SiteUnit& u, c
 #pragma unroll
         for (int i = 0; i < TA; ++i)
 #pragma unroll
-          for (int e = 0; e < TC; ++e) cmac<T>(x[i][e], q[i], g[e]);
+          for (int e = 0; e < TC; ++e) cmac<T>(acc[i][e][u4], q[i], g[e]);
+      };
+      int k = 0;
+      for (; k + 3 < K; k += 4) {
+#pragma unroll
+        for (int u4 = 0; u4 < 4; ++u4) step(k + u4, u4 % U);
       }
+      for (; k < K; ++k) step(k, 0);
+#pragma unroll
+      for (int i = 0; i < TA; ++i)
+#pragma unroll
+        for (int e = 0; e < TC; ++e) x[i][e] = sum_parts<U>(acc[i][e]);
       if (jb.nnz > 0) {
 #pragma unroll
         for (int i = 0; i < TA; ++i)
@@ -541,29 +558,37 @@ __device__ __noinline__ bool op_env_site(const KernelParams& P, Team& tm, const 
           const V *q0 = qs + a0 * sp.Cp, *q1 = qs + a1 * sp.Cp;
           const V* ys = Y + b * Yblk + sl * u.A * Yrow;
           const V *y0 = ys + p0 * Yrow, *y1 = ys + p1 * Yrow;
-          V s00, s01, s10, s11;
-          s00.x = s00.y = s01.x = s01.y = s10.x = s10.y = s11.x = s11.y = (T)0;
+          constexpr int U = kMixed ? 4 : 1;
+          V s[4][U];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int u4 = 0; u4 < U; ++u4) s[q][u4].x = s[q][u4].y = (T)0;
           auto cj = [](V& s, V q, V y) {  // s += conj(q) y
             s.x = fma(q.x, y.x, fma(q.y, y.y, s.x));
             s.y = fma(q.x, y.y, fma(-q.y, y.x, s.y));
           };
-          for (int c = sub; c < sp.Dc; c += ksp) {
+          auto step = [&](int c, int u4) {
             const V u0 = q0[c], u1 = q1[c], w0 = y0[c], w1 = y1[c];
-            cj(s00, u0, w0);
-            cj(s01, u0, w1);
-            cj(s10, u1, w0);
-            cj(s11, u1, w1);
-          }
-          auto add = [&](E& e, V s) {
-            if constexpr (kMixed)
-              e = A::c(A::add(A::re(e), make_float2(s.x, 0.f)), A::add(A::im(e), make_float2(s.y, 0.f)));
-            else
-              e = A::c(A::add(A::re(e), s.x), A::add(A::im(e), s.y));
+            cj(s[0][u4], u0, w0);
+            cj(s[1][u4], u0, w1);
+            cj(s[2][u4], u1, w0);
+            cj(s[3][u4], u1, w1);
           };
-          add(acc[0], s00);
-          add(acc[1], s01);
-          add(acc[2], s10);
-          add(acc[3], s11);
+          int c = sub;
+          for (; c + 3 * ksp < sp.Dc; c += 4 * ksp) {
+#pragma unroll
+            for (int u4 = 0; u4 < 4; ++u4) step(c + u4 * ksp, u4 % U);
+          }
+          for (; c < sp.Dc; c += ksp) step(c, 0);
+          auto add = [&](E& e, V t) {
+            if constexpr (kMixed)
+              e = A::c(A::add(A::re(e), make_float2(t.x, 0.f)), A::add(A::im(e), make_float2(t.y, 0.f)));
+            else
+              e = A::c(A::add(A::re(e), t.x), A::add(A::im(e), t.y));
+          };
+#pragma unroll
+          for (int q = 0; q < 4; ++q) add(acc[q], sum_parts<U>(s[q]));
         }
       for (int o = ksp >> 1; o > 0; o >>= 1)
 #pragma unroll

@@ -93,6 +93,24 @@ __device__ __forceinline__ void cmac(typename C2<T>::t& acc, typename C2<T>::t a
   acc.y = fma(a.x, b.y, acc.y);
   acc.y = fma(a.y, b.x, acc.y);
 }
+// Sum of U partial sums.  In FP32 the products of a leg and the projections keep four accumulators
+// per output (every fourth term each), as mode_dot does: with one, the rounding of a chain of 20 to
+// 64 additions made the errors against FP64 references 1.1 to 1.4 times as large (one step of 4 x 3
+// stars of D 16 and 20, two steps of 8-site chains of D 24; geometric means over 24 to 64 seeds;
+// 0.9 to 1.05 now).  It costs 0.4 to 3.4 %: 25-site chain 44.2 -> 45.7 ms, 4 x 20 star 56.1 -> 57.1, 8 x 60 ER tree
+// 348.3 -> 349.7.
+template <int U, typename V>
+__device__ __forceinline__ V sum_parts(const V* a) {
+  V r = a[0];
+  if constexpr (U == 2) {
+    r.x += a[1].x;
+    r.y += a[1].y;
+  } else if constexpr (U == 4) {
+    r.x += a[1].x + (a[2].x + a[3].x);
+    r.y += a[1].y + (a[2].y + a[3].y);
+  }
+  return r;
+}
 
 // ------------------------------------------------------------------ teams
 struct Team {
@@ -753,8 +771,9 @@ __device__ __forceinline__ void tile_rows(const typename C2<T>::t* M, int D, int
   for (int it = threadIdx.x; it < nrg * ncg; it += NT) {
     const int rg = fdivu(it, ncg, inv_g), c0 = it - rg * ncg, i0 = rg * TA;
     int base[TC];
+    constexpr int U = TA * TC > 4 ? 2 : 4;  // (more would spill)
     const V* row[TA];
-    V acc[TA][TC];
+    V acc[TA][TC][U];
 #pragma unroll
     for (int q = 0; q < TC; ++q) {
       const int c = min(c0 + q * ncg, nc - 1), hi = fdivu(c, st, inv_st);
@@ -764,10 +783,11 @@ __device__ __forceinline__ void tile_rows(const typename C2<T>::t* M, int D, int
     for (int i = 0; i < TA; ++i) {
       row[i] = M + min(i0 + i, D - 1) * D;
 #pragma unroll
-      for (int q = 0; q < TC; ++q) acc[i][q].x = acc[i][q].y = (T)0;
+      for (int q = 0; q < TC; ++q)
+#pragma unroll
+        for (int u = 0; u < U; ++u) acc[i][q][u].x = acc[i][q][u].y = (T)0;
     }
-#pragma unroll 4
-    for (int k = 0; k < D; ++k) {
+    auto step = [&](int k, int u) {
       V m[TA], v[TC];
 #pragma unroll
       for (int i = 0; i < TA; ++i) m[i] = row[i][k];
@@ -776,15 +796,21 @@ __device__ __forceinline__ void tile_rows(const typename C2<T>::t* M, int D, int
 #pragma unroll
       for (int i = 0; i < TA; ++i)
 #pragma unroll
-        for (int q = 0; q < TC; ++q) cmac<T>(acc[i][q], m[i], v[q]);
+        for (int q = 0; q < TC; ++q) cmac<T>(acc[i][q][u], m[i], v[q]);
+    };
+    int k = 0;
+    for (; k + 3 < D; k += 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) step(k + u, u % U);
     }
+    for (; k < D; ++k) step(k, 0);
 #pragma unroll
     for (int i = 0; i < TA; ++i)
 #pragma unroll
       for (int q = 0; q < TC; ++q)
         if (i0 + i < D && c0 + q * ncg < nc) {
           V* o = out + base[q] + (i0 + i) * st;
-          V r = acc[i][q];
+          V r = sum_parts<U>(acc[i][q]);
           if (add) {
             r.x += o->x;
             r.y += o->y;
@@ -1708,31 +1734,40 @@ __device__ __noinline__ bool project_rows(const KernelParams& P, Team& tm, const
         const int ta = fdivu(it, h, inv_h);
         const int a0 = 2 * ta, a1 = min(a0 + 1, D - 1), p0 = 2 * (it - ta * h), p1 = min(p0 + 1, D - 1);
         const V *q0 = Qs + a0 * RP, *q1 = Qs + a1 * RP, *y0 = Ys + p0 * RP, *y1 = Ys + p1 * RP;
-        V s[4];
+        constexpr int U = std::is_same<T, double>::value ? 1 : 4;
+        V s[4][U];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) s[q].x = s[q].y = (T)0;
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int u = 0; u < U; ++u) s[q][u].x = s[q][u].y = (T)0;
         auto cj = [](V& e, V q, V y) {  // e += conj(q) y
           e.x = fma(q.x, y.x, fma(q.y, y.y, e.x));
           e.y = fma(q.x, y.y, fma(-q.y, y.x, e.y));
         };
-#pragma unroll 4
-        for (int r = 0; r < nr; ++r) {
+        auto step = [&](int r, int u) {
           const V u0 = q0[r], u1 = q1[r], w0 = y0[r], w1 = y1[r];
-          cj(s[0], u0, w0);
-          cj(s[1], u0, w1);
-          cj(s[2], u1, w0);
-          cj(s[3], u1, w1);
+          cj(s[0][u], u0, w0);
+          cj(s[1][u], u0, w1);
+          cj(s[2][u], u1, w0);
+          cj(s[3][u], u1, w1);
+        };
+        int r = 0;
+        for (; r + 3 < nr; r += 4) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) step(r + u, u % U);
         }
+        for (; r < nr; ++r) step(r, 0);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int a = a0 + (q >> 1), p = p0 + (q & 1);
           if (a >= D || p >= D) continue;
           E& e = mine[b * D2 + a * D + p];
           E o = r0 == rb ? A::c(A::zero(), A::zero()) : e;
+          const V t = sum_parts<U>(s[q]);
           if constexpr (std::is_same<T, double>::value)
-            o = A::c(A::add(A::re(o), s[q].x), A::add(A::im(o), s[q].y));
+            o = A::c(A::add(A::re(o), t.x), A::add(A::im(o), t.y));
           else
-            o = A::c(A::add(A::re(o), make_float2(s[q].x, 0.f)), A::add(A::im(o), make_float2(s[q].y, 0.f)));
+            o = A::c(A::add(A::re(o), make_float2(t.x, 0.f)), A::add(A::im(o), make_float2(t.y, 0.f)));
           e = o;
         }
       }
