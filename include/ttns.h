@@ -292,6 +292,10 @@ typedef struct {
 } ttns_counters;
 ttns_status ttns_get_counters(ttns_tree* tree, ttns_counters* out);
 
+/* CTAs of the tree set's sweep kernel on one SM: 1, or 2 for a set of many small trees that is
+ * run two at a time (never when ttns_options.grid_ctas is given). */
+ttns_status ttns_ctas_per_sm(ttns_tree* tree, int* out);
+
 /* Node tensor access (layout: legs [parent] + [children in order] + [physical],
  * row-major).  ttns_node_info gives the number of nodes of tree tree_idx when
  * node < 0, else node's leg count and dims (dims: up to 8 ints). */

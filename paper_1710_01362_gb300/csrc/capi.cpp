@@ -1443,6 +1443,12 @@ extern "C" ttns_status ttns_get_counters(ttns_tree* t, ttns_counters* out) {
   return TTNS_OK;
 }
 
+extern "C" ttns_status ttns_ctas_per_sm(ttns_tree* t, int* out) {
+  if (!t || !out) return fail(TTNS_E_INVALID, "NULL argument");
+  *out = t->pair ? 2 : 1;
+  return TTNS_OK;
+}
+
 extern "C" ttns_status ttns_node_info(ttns_tree* t, int tree_idx, int node, int* n_legs, int* dims, int* n_nodes) {
   if (!t) return fail(TTNS_E_INVALID, "tree is NULL");
   if (tree_idx < 0 || tree_idx >= (int)t->C.trees.size()) return fail(TTNS_E_INVALID, "tree_idx out of range");

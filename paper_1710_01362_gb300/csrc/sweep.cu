@@ -94,11 +94,11 @@ __device__ __forceinline__ void cmac(typename C2<T>::t& acc, typename C2<T>::t a
   acc.y = fma(a.y, b.x, acc.y);
 }
 // Sum of U partial sums.  In FP32 the products of a leg and the projections keep four accumulators
-// per output (every fourth term each), as mode_dot does: with one, the rounding of a chain of 20 to
+// per output (every fourth term each), as mode_dot does: with one, the rounding of a chain of 16 to
 // 64 additions made the errors against FP64 references 1.1 to 1.4 times as large (one step of 4 x 3
 // stars of D 16 and 20, two steps of 8-site chains of D 24; geometric means over 24 to 64 seeds;
-// 0.9 to 1.05 now).  It costs 0.4 to 3.4 %: 25-site chain 44.2 -> 45.7 ms, 4 x 20 star 56.1 -> 57.1, 8 x 60 ER tree
-// 348.3 -> 349.7.
+// 0.8 to 1.07 now).  They cost 0.4 to 3.4 %: 25-site chain 44.2 -> 45.7 ms, 4 x 20 star 56.1 ->
+// 57.1, 8 x 60 ER tree 348.3 -> 349.7.
 template <int U, typename V>
 __device__ __forceinline__ V sum_parts(const V* a) {
   V r = a[0];

@@ -30,7 +30,7 @@ EXPORTS = [
     "ttns_chain_ohmic", "ttns_chain_from_modes", "ttns_plan", "ttns_selftest_wait_timeout",
     "ttns_rho_from_root_noalloc", "ttns_autotune", "ttns_selftest_tc_gemm", "ttns_mlp_gemm", "ttns_mlp_colsum",
     "ttns_mlp_diff", "ttns_mlp_adam", "ttns_mlp_status", "ttns_energy_surfaces", "ttns_bond_entropies",
-    "ttns_cluster_modes", "ttns_grow_bonds", "ttns_adapt_bonds",
+    "ttns_cluster_modes", "ttns_grow_bonds", "ttns_adapt_bonds", "ttns_ctas_per_sm",
 ]
 
 
@@ -106,6 +106,7 @@ def lib():
         L.ttns_cluster_modes.argtypes = [C.c_int, C.c_int, dp, C.c_int, ip, C.c_int, ip, dp, dp, ip]
         L.ttns_populations_device.argtypes = [C.c_void_p, C.c_void_p]
         L.ttns_get_counters.argtypes = [C.c_void_p, C.POINTER(Counters)]
+        L.ttns_ctas_per_sm.argtypes = [C.c_void_p, C.POINTER(C.c_int)]
         L.ttns_node_info.argtypes = [C.c_void_p, C.c_int, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int),
                                      C.POINTER(C.c_int)]
         L.ttns_get_node.argtypes = [C.c_void_p, C.c_int, C.c_int, dp, C.c_size_t]
@@ -439,6 +440,12 @@ class Tree:
                 "env_phases_grid": dict(zip(env_names, [c.env_phase_seconds[1][k] for k in range(4)])),
                 "tc_phases": dict(zip(["staging", "mma", "readback", "write"], [c.tc_phase_seconds[k] for k in range(4)])),
                 "launch_fallbacks": c.launch_fallbacks}
+
+    def ctas_per_sm(self) -> int:
+        """CTAs of the sweep kernel on one SM (2 for sets of many small trees)."""
+        n = C.c_int()
+        _check(lib().ttns_ctas_per_sm(self.h, C.byref(n)))
+        return n.value
 
     def n_nodes(self, k: int = 0) -> int:
         n = C.c_int()
