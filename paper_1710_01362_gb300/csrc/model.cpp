@@ -832,6 +832,21 @@ Compiled compile_trees(const std::vector<TreeInput>& inputs, bool batched, int g
     const HostTree kin = kinetic_tree(C.host[i], inputs[i]);
     TreeCompiler kc(kin, C, (int)i, batched, grid_threshold, qr_grid_threshold);
     kc.compile_operator(td.node0, &td.obs_first, &td.obs_count, &td.teff_terms);
+    if (i == 0 && inputs.size() > 1) {
+      // Room for the set by the size of its first tree (at most 2 GB a table; other trees may be
+      // larger or smaller): growing the tables step by step, each time with a copy into fresh
+      // pages, was a third of the compilation of 304 ER trees.
+      auto room = [&](auto& v) {
+        const size_t most = (size_t(1) << 31) / sizeof(v[0]);
+        v.reserve(std::max(v.size(), std::min(most, v.size() * inputs.size())));
+      };
+      room(C.pool_init);
+      room(C.terms);
+      room(C.lists);
+      room(C.chans);
+      room(C.prog);
+      room(C.nodes);
+    }
   }
   // trajectory buffers at the end of the pool
   for (auto& td : C.trees) {
