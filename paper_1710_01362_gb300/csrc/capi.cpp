@@ -620,13 +620,13 @@ static ttns_status device_init(ttns_tree* t) try {
   std::stable_sort(order.begin(), order.end(),
                    [&](int a, int b) { return C.trees[a].prog_count > C.trees[b].prog_count; });
   // Two CTAs per SM where it shortens the whole set: beside another one a cluster takes 1.16
-  // (four-CTA teams) to 1.6 times as long (one-CTA teams), so the set has to gain more than
-  // that from twice the clusters.  Not for tensors from the size at which the tensor-core
+  // (four-CTA teams) to 1.6 times as long (one-CTA teams); the rule asks every team for the larger
+  // factor from twice the clusters.  Not for tensors from the size at which the tensor-core
   // products start, nor where a plan or the QR's buffers need more than half the shared memory:
   // FP64 chains of D 12-24 on one CTA took 2906 ms instead of 1960 when their plans did not fit.
-  // Measured, one CTA per SM against two: 256 chains on four CTAs 218 and 136 ms, on eight 439 and
-  // 214; 304 ER trees of D 8 91 and 73 ms (TF32X3), 184 and 133 (FP64); 64 chains on four CTAs
-  // (36 clusters fit) 99 and 102.
+  // Measured, one CTA per SM against two, the first and the fourth step of a run: 256 chains on
+  // four CTAs 189 and 230 ms against 109 and 140, on eight 390 and 469 against 189 and 231; 304 ER
+  // trees of D 8 85 and 95 against 69 and 76 (TF32X3), 169 and 192 against 123 and 139 (FP64).
   if (t->batched && o.grid_ctas <= 0 && C.max_node < kPairNode && C.max_D <= kPairD) {
     std::vector<double> cost;
     for (int k : order) cost.push_back(C.trees[k].prog_count);

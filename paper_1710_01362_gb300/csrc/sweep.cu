@@ -52,7 +52,6 @@ namespace pair {
 #define ST_LAUNCH 3       // the launch did not have the cluster shape / shared memory it was planned for
 
 __constant__ double c_inv[256];       // 1/n, c_inv[0] = 0
-__constant__ double c_invfact[128];   // 1/n!
 
 // ------------------------------------------------------------------ complex helpers
 template <typename T> struct C2;
@@ -665,9 +664,6 @@ __device__ __forceinline__ void team_reduce_vec(Team& tm, const double* mine, in
     tm.parity ^= 1;
   }
   __syncthreads();
-}
-__device__ void team_reduce_vec(Team& tm, const double* mine, double* out, int nval) {
-  team_reduce_vec(tm, mine, nval, [&](int k, double v) { out[k] = v; });
 }
 
 #include "krylov.cuh"
@@ -2123,9 +2119,10 @@ __device__ __forceinline__ unsigned sreg_dynamic_smem_size() {
 // The two-CTA instance: what bounds batches of small trees is latency (FP64 chains, cluster
 // barriers, scalar steps on one warp), and a second tree on the SM fills the waits.  It has half
 // the registers and shared memory and no tensor memory (its trees are below the size at which
-// the tensor-core products start).  One step of 256 chains of 10 to 40 sites on four-CTA teams
-// (TF32X3): 327 ms before (trees in order, one per cluster at a time), 218 with the longest first
-// on whichever cluster is free, 136 with two CTAs per SM.
+// the tensor-core products start).  256 chains of 10 to 40 sites on four-CTA teams (TF32X3): 327 ms
+// a step with the trees in order, one per cluster at a time, 218 with the longest first on
+// whichever cluster is free, 136 with two CTAs per SM (third step of a run; the first takes a fifth
+// less).
 __global__ void __launch_bounds__(NT, SWEEP_CTAS) k_sweep(KernelParams P, int phase) {
   // Launch self-check before any barrier or distributed-shared-memory access: the
   // interpreter addresses cluster peers by rank and stages operands up to smem_bytes, so a
@@ -2137,7 +2134,7 @@ __global__ void __launch_bounds__(NT, SWEEP_CTAS) k_sweep(KernelParams P, int ph
     if (threadIdx.x == 0 && blockIdx.x == 0) set_status(P.ctl, ST_LAUNCH, 300, (int)ncta);
     return;
   }
-  // tensor memory for the split-precision contractions (one 128-column accumulator per CTA)
+  // tensor memory for the split-precision contractions (all 512 columns: one accumulator per K step)
   const bool tc_on = SWEEP_CTAS == 1 && (P.precision == 1 || P.precision == 2);
   if (threadIdx.x == 0) s_tc.on = 0;
   if (tc_on) {
@@ -2361,14 +2358,10 @@ static bool g_tables_set = false;
 
 static cudaError_t upload_constants() {
   if (g_tables_set) return cudaSuccess;
-  double inv[256], invf[128];
+  double inv[256];
   inv[0] = 0.0;
   for (int k = 1; k < 256; ++k) inv[k] = 1.0 / k;
-  invf[0] = 1.0;
-  for (int k = 1; k < 128; ++k) invf[k] = invf[k - 1] / k;
-  cudaError_t e = cudaMemcpyToSymbol(c_inv, inv, sizeof(inv));
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyToSymbol(c_invfact, invf, sizeof(invf));
+  const cudaError_t e = cudaMemcpyToSymbol(c_inv, inv, sizeof(inv));
   if (e == cudaSuccess) g_tables_set = true;
   return e;
 }
