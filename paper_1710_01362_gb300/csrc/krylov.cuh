@@ -25,6 +25,7 @@ struct KrylovShared {
   double ratio;
   double s_done;
   int fused, check, conv, again;
+  int full;                     // the last check left the expansion of its m and s in ure, uim
 };
 __shared__ KrylovShared s_ks;
 
@@ -223,13 +224,15 @@ __device__ __noinline__ void texp_warp(const double* a, const double* b, int m, 
 // Krylov matrices of m = 2 to 32 against FP64; beyond 30 m it can be off by any factor).  Within 1 %
 // or 5 % of the tolerance, with wider spectra and for smaller tolerances the FP64 expansion decides:
 // one step more or less changes what is left below the tolerance, and the QR's null decisions can
-// amplify that.  (With 12 m as the limit, 256 chains of up to 40 sites took 4.8 % longer.)
+// amplify that.  (With 12 m as the limit, 256 chains of up to 40 sites took 4.8 % longer.)  `full`:
+// ure and uim hold the FP64 expansion.
 __device__ __noinline__ bool krylov_small(const KrylovShared& ks, int m, double s, double tol, double* ure,
-                                          double* uim, bool* nonfinite) {
+                                          double* uim, bool* nonfinite, bool* full) {
   const int lane = threadIdx.x & 31;
   const double bn = ks.beta[m];
   ChebSetup cs = cheb_setup(ks.alpha, ks.beta, m, fabsf((float)s));
   *nonfinite = false;
+  *full = false;
   const float width = cs.z * cs.z / (float)m;
   if (width <= 20.f && tol >= 1e-15 * bn) {
     cheb_order(cs, cs.z);
@@ -266,28 +269,34 @@ __device__ __noinline__ bool krylov_small(const KrylovShared& ks, int m, double 
     if (err >= (1.0 + margin) * tol) return false;
   }
   texp_warp(ks.alpha, ks.beta, m, s, ure, uim);
+  *full = true;
   const double r = ure[m - 1], i = uim[m - 1];
   const double err = bn * sqrt(r * r + i * i);
   if (!(err == err)) *nonfinite = true;
   return err <= tol || !(bn > 0.0);
 }
 __device__ __forceinline__ void krylov_check(KrylovShared& ks, int m, double s, double tol) {
-  bool bad;
-  const bool ok = krylov_small(ks, m, s, tol, ks.ure, ks.uim, &bad);
-  if ((threadIdx.x & 31) == 0) ks.conv = bad ? 2 : (ok ? 1 : 0);
+  bool bad, full;
+  const bool ok = krylov_small(ks, m, s, tol, ks.ure, ks.uim, &bad, &full);
+  if ((threadIdx.x & 31) == 0) {
+    ks.conv = bad ? 2 : (ok ? 1 : 0);
+    ks.full = full;
+  }
 }
 // After the last step (warp 0): the time that the space covers (s, or with `halve` the largest
-// s / 2^k, k <= 30, that reaches the tolerance) and the coefficients of the result.
+// s / 2^k, k <= 30, that reaches the tolerance) and the coefficients of the result, which a check in
+// FP64 has left behind.  (A step ends with a check: at the last m of a space at the latest.)
 __device__ __noinline__ void krylov_exp(KrylovShared& ks, int m, double s, double tol, bool halve) {
+  const int lane = threadIdx.x & 31;
+  bool full = ks.full != 0;
   if (halve) {
     for (int k = 0; k < 30; ++k) {
       s *= 0.5;
       bool bad;
-      if (krylov_small(ks, m, s, tol, ks.ure, ks.uim, &bad)) break;
+      if (krylov_small(ks, m, s, tol, ks.ure, ks.uim, &bad, &full)) break;
     }
   }
-  texp_warp(ks.alpha, ks.beta, m, s, ks.ure, ks.uim);
-  const int lane = threadIdx.x & 31;
+  if (!full) texp_warp(ks.alpha, ks.beta, m, s, ks.ure, ks.uim);
   if (lane < m) {
     const double sc = ks.beta0 * ks.scale[lane];
     ks.ure[lane] *= sc;
