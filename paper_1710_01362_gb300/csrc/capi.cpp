@@ -1622,8 +1622,11 @@ ttns_status adopt_tables(ttns_tree* t, const std::vector<double2>& pool) {
   if (changed.empty()) return TTNS_OK;
   for (const auto& c : changed) std::copy_n(pool.begin() + c.first, c.second, C.pool_init.begin() + c.first);
   build_site_plans(t, t->grid, t->P.smem_bytes);
-  t->allocs.erase(std::find(t->allocs.begin(), t->allocs.end(), (void*)t->d_sites));
-  cudaFree(t->d_sites);
+  const auto old = std::find(t->allocs.begin(), t->allocs.end(), (void*)t->d_sites);
+  if (old != t->allocs.end()) {
+    cudaFree(*old);
+    t->allocs.erase(old);
+  }
   ttns_status s = upload(t, &t->d_sites, t->sites);
   if (s != TTNS_OK) {  // the general forms, which need no plan
     t->d_sites = nullptr;

@@ -24,6 +24,7 @@
 #include <cmath>
 #include <functional>
 #include <map>
+#include <new>
 #include <stdexcept>
 #include <string>
 
@@ -838,7 +839,10 @@ Compiled compile_trees(const std::vector<TreeInput>& inputs, bool batched, int g
       // pages, was a third of the compilation of 304 ER trees.
       auto room = [&](auto& v) {
         const size_t most = (size_t(1) << 31) / sizeof(v[0]);
-        v.reserve(std::max(v.size(), std::min(most, v.size() * inputs.size())));
+        try {
+          v.reserve(std::max(v.size(), std::min(most, v.size() * inputs.size())));
+        } catch (const std::bad_alloc&) {  // the tables then grow as they need to
+        }
       };
       room(C.pool_init);
       room(C.terms);
