@@ -54,9 +54,12 @@ typedef enum {
 
 /* Precision of the contractions (H_eff / H_bond applications and environment updates).  In
  * every mode the Krylov basis and recurrence, the small exponential and the observables are
- * FP64.  The QR bond steps and the gauge absorbs are FP64 in TTNS_FP64 and double-single
+ * FP64 (whether a Krylov space suffices is estimated in FP32 first; the FP64 exponential decides
+ * wherever that estimate is not certain).  The QR bond steps, the gauge absorbs and the sums of
+ * environment updates over slices, blocks of rows and CTAs are FP64 in TTNS_FP64 and double-single
  * (unevaluated sums of two floats, 48-bit significand, error-free transformations; about
- * 2^-44 relative per operation, FP32's exponent range) in the other modes.
+ * 2^-44 relative per operation, FP32's exponent range) in the other modes; environment updates whose
+ * outputs are split over the CTAs add their runs of 64 rows in FP64 in every mode.
  *   TTNS_FP64    every contraction in FP64;
  *   TTNS_TF32X3  split-precision tensor cores: the H_eff applications of tensors of at least 4096
  *                elements whose terms have one dense factor each, other than chain sites and

@@ -15,7 +15,7 @@
 // to the CTAs that read its slices, through distributed shared memory (cluster teams) or a
 // slice-major copy in global memory (the grid team).
 // Forward exponential of a 40 x 40 x 20 tensor, whole grid, about four applications: 190 us per
-// operation before, 102 now (BF16X3 mode); FP64, about eight applications: 1500 and 660.
+// operation before, 103 now (BF16X3 mode); FP64, about eight applications: 1500 and 660.
 //
 // The plan (legs, jobs, split, layout: SitePlan) comes from the host: worked out by one thread of
 // every CTA it took 6 us per operation.

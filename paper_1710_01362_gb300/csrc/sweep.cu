@@ -682,10 +682,10 @@ __device__ __forceinline__ void team_reduce_vec(Team& tm, const double* mine, in
 // factor on its result: element by element the operand loads are the bound (two shared-memory
 // or L2 words per multiply-add).  Root of a star of four chains (20^4 x 5, two of the couplings
 // with three entries a row, which kept it from being tiled), whole grid, TF32X3 mode: 5760 us per
-// exponential before, 3410 now.  In FP64 the FP64 pipe is the bound in either form (18.9 ms
-// element by element, 20.5 by products), so there, and where three tiles (input, sum, product)
-// do not fit in shared memory, a tile's terms are taken element by element, without two-stage
-// terms.
+// exponential before, 3500 now (3250 with one accumulator).  In FP64 the FP64 pipe is the bound in
+// either form (18.9 ms element by element, 20.5 by products), so there, and where three tiles
+// (input, sum, product) do not fit in shared memory, a tile's terms are taken element by element,
+// without two-stage terms.
 struct TiledApply {
   NodeDesc ta, tb;                  // the tile tensors of the two passes
   int h;
@@ -1457,10 +1457,10 @@ __device__ __noinline__ void op_expm(const KernelParams& P, Team& tm, const Inst
   constexpr bool kShadow = !std::is_same<T, double>::value;
   // tensor-core apply (split precision) for nodes whose terms have one dense factor each; its
   // operand tiles take the dynamic shared memory, so nothing staged there is used
-  // (a large root's tiles first: 2980 us per exponential at 20^4 x 5, the tensor cores 4210 in
-  // TF32X3 and 3550 in BF16X3, where splitting the operands is the bound; at 14^4 x 5 980 us, there
-  // 980 and 1030.  With fewer tiles than CTAs the tensor cores are ahead: 400 us at 20^3 x 5, by
-  // tiles 580)
+  // (a large root's tiles first: 2980 us per exponential at 20^4 x 5, 8 % more since their products
+  // keep several accumulators; the tensor cores 4210 in TF32X3 and 3550 in BF16X3, where splitting
+  // the operands is the bound; at 14^4 x 5 980 us, there 980 and 1030.  With fewer tiles than CTAs
+  // the tensor cores are ahead: 400 us at 20^3 x 5, by tiles 580)
   V* xt = nullptr;
   bool tiled = false, fibres = false, use_tc = false;
   if constexpr (kShadow)
